@@ -157,11 +157,9 @@ int muca_set_launch(ea_ctx *ctx, int persistent, uint64_t sweeps_per_launch, int
  *   c(x) = x mod 3 except c(L-1) = 1 when L = 1 (mod 3)), each in lexicographic order; the
  *   j-th colour-c site of a row takes word j&3 of call (4 row + j/4, t, rid, (5 + c) | stream << 8).
  *   No two sites of a class are neighbours, so each attempt's class is fixed when its class
- *   begins.  One kernel runs it for every L, one lane per chain in the tiles of the lexicographic
- *   kernel (the tile widths of muca_set_tile_width apply; odd L has three colour passes and
- *   rows with different numbers of colour sites, padded with attempts that move nothing): one
- *   candidate-threshold pair per attempt instead of two classes' worth, the faster order for
- *   L <= 8.
+ *   begins.  Two kernels run it, for every L, with the same results: one warp per chain, and one
+ *   lane per chain for batches of full tiles that fill the GPU; the library takes the one it
+ *   estimates to be faster for the context's tiles.  The faster order for small and middle batches.
  * chains_per_cta: 0 or one of 1, 2, 4, 8 (kept for callers of an earlier form of this call; it
  * has no effect).  Applies from the next muca_run_sweeps or graph capture; the order is not part
  * of a snapshot.  EA_EINVAL for an unknown order or count. */
@@ -170,12 +168,12 @@ int muca_set_sweep_order(ea_ctx *ctx, int order, int chains_per_cta);
 /* a8 -- chains per tile for chains of linear size L added afterwards (ea_init_disorder):
  * width 32 (the default, every L), 16 (3D, L = 7, 8), or, for chains swept in the colour order
  * only, 16 (3D, L = 4, 5, 6), 8 (3D, L = 4..10) and 4 (3D, L = 11, 12); muca_run_sweeps in the
- * lexicographic order refuses tiles of a width that kernel lacks (EA_EINVAL).  A tile is one
- * warp; with width W < 32 each of its W chains runs on 32/W lanes side by side, so the tile needs
- * W/32 of the shared memory of a full one: at L >= 7 the acceptance thresholds then fit in shared
- * memory instead of being read through L1, and at every L a batch spreads over more SMs with less
- * producer work on each; each chain runs faster, the SM holds fewer chains.  Narrow tiles suit
- * batches with fewer chains than the GPU can hold; results do not depend on the width.
+ * lexicographic order refuses tiles of a width that kernel lacks (EA_EINVAL).  In the
+ * lexicographic order a tile is one warp; with width W < 32 each of its W chains runs on 32/W lanes
+ * side by side, so the tile needs W/32 of the shared memory of a full one: at L >= 7 the acceptance
+ * thresholds then fit in shared memory instead of being read through L1.  In the colour order the
+ * width matters little: a chain has a warp of its own unless the batch fills the GPU.  Narrow tiles
+ * suit batches with fewer chains than the GPU can hold; results do not depend on the width.
  * EA_EINVAL for a width not available at this L. */
 int muca_set_tile_width(ea_ctx *ctx, int L, int width);
 
@@ -183,7 +181,8 @@ int muca_set_tile_width(ea_ctx *ctx, int L, int width);
  * (*smem_bytes, may be NULL) and whether the thresholds live in shared memory
  * (*thresholds_in_smem, may be NULL).  EA_EINVAL for a width not available at this L. */
 int muca_get_tile_width(int dim, int L, int width, size_t *smem_bytes, int *thresholds_in_smem);
-/* The same for the colour-order kernel (muca_set_sweep_order). */
+/* The same for the colour order's one-warp-per-chain kernel (muca_set_sweep_order): shared memory
+ * of a chain's block; the thresholds around its current bin are in it. */
 int muca_get_tile_width_colour(int dim, int L, int width, size_t *smem_bytes, int *thresholds_in_smem);
 
 /* a8 / a9 -- every tile of linear size L runs multiplier x the requested sweeps in each

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -359,9 +360,9 @@ extern "C" int ea_init_disorder(ea_ctx *ctx, int dim, int L, int n, uint32_t rid
     // the tile width: the configured one where either sweep kernel has it (8 and 4 only the
     // colour-order kernel), else 32
     const int Wc = ctx->tile_width[L];
-    const bool lex_w = sweep_width_supported(dim, L, Wc), col_w = checker_smem_bytes(dim, L, Wc) > 0;
+    const bool lex_w = sweep_width_supported(dim, L, Wc), col_w = colour_width_supported(dim, L, Wc);
     const int W = (lex_w || col_w) ? Wc : kTile;
-    const size_t need = std::max(lex_w || W == kTile ? sweep_smem_bytes(dim, L, W) : 0, checker_smem_bytes(dim, L, W));
+    const size_t need = std::max(lex_w || W == kTile ? sweep_smem_bytes(dim, L, W) : 0, walk_smem_bytes(dim, L));
     if (need > (size_t)smem_optin)
         return fail(EA_EINVAL, "L=%d needs %zu bytes of shared memory per block, the device allows %d", L, need,
                     smem_optin);
@@ -634,23 +635,50 @@ extern "C" int muca_set_eg(ea_ctx *ctx, int chain0, int n, const int32_t *e_g) {
     return EA_OK;
 }
 
-// The colour order runs in the checkerboard kernels (one lane per chain in the tiles of the
-// lexicographic kernel; three colour passes for odd L, a kernel of their own); the shared memory
-// for the context's tiles and which kernel-form classes occur (bit 0 even, bit 1 odd L, bit 2 the
-// small even sizes' narrow tiles).
-static int colour_launch(ea_ctx *ctx, size_t *ck_smem_out, int *parities) {
-    int optin = 0;
-    EA_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
-    size_t ck = 0;
-    int par = 0;
+// The colour order has two kernels with the same results: one warp per chain (muca_walk.cu: 22 cycles
+// per attempt of a chain that has a scheduler to itself, and about 11 issue cycles per attempt, so
+// slower as chains share schedulers) and one lane per chain (muca_checker.cu: 45 to 220 cycles by
+// size and tile width, the same for every chain of a block, one block per SM).  The plan estimates
+// both times of a launch, in cycles, and takes the shorter:
+//   walk:    f (23 a_max + 10.2 sum of a / schedulers), a = attempts of a chain, f by L; fitted to
+//            512 .. 16384 chains of every L between hot chains (first iterations, one third more) and
+//            cold ones (production, one fifth less);
+//   checker: cycles(L, width) a per wave of one block per SM, as measured.
+// The line lies near 2000 to 4000 chains in full tiles.  Both sides, attempts/ns (walk hot .. cold /
+// checker): L = 8 in tiles of 16, 1024 chains 53 .. 76 / 45, 2048 69 .. 95 / 89, 4096 80 .. 109 / 89;
+// L = 6 in full tiles, 1024 47 / 33, 2048 63 .. 70 / 65, 4096 73 / 130; L = 4, 2048 57 / 42, 4096 65 / 84.
+struct ColourPlan {
+    bool walk = true;
+    size_t smem = 0;
+    int max_width = 0, parities = 0;
+};
+
+static ColourPlan colour_plan(const ea_ctx *ctx) {
+    static const double f_walk[13] = {0, 0, 0, 4.1, 1.27, 1.4, 1.09, 1.13, 1.0, 1.15, 1.28, 1.28, 1.18};
+    static const double c_full[13] = {0, 0, 0, 220, 100, 146, 64.5, 155, 101, 125, 104, 137, 111};
+    static const double c_half[13] = {0, 0, 0, 0, 79, 113, 60.5, 83, 47.5, 0, 0, 0, 0};
+    ColourPlan walk, checker;
+    checker.walk = false;
+    bool have = true;  // the checker kernel has every tile's width
+    double w_max = 0, w_sum = 0, c_max = 0, c_sum = 0;
     for (const TileDesc &td : ctx->tiles) {
-        ck = std::max(ck, checker_smem_bytes(td.dim, td.L, td.width));
-        par |= checker_parity_class(td.dim, td.L, td.width);
+        const double a = (double)td.V * std::max(1, td.sweep_mul), f = td.dim == 3 ? f_walk[td.L] : 1.5;
+        walk.smem = std::max(walk.smem, walk_smem_bytes(td.dim, td.L));
+        walk.max_width = std::max(walk.max_width, (int)td.width);
+        w_max = std::max(w_max, f * a);
+        w_sum += f * a * td.n_active;
+        const size_t ck = checker_smem_bytes(td.dim, td.L, td.width);
+        have = have && ck > 0;
+        checker.smem = std::max(checker.smem, ck);
+        checker.parities |= checker_parity_class(td.dim, td.L, td.width);
+        const double c = a * (td.dim == 3 ? (td.width == 32 ? c_full[td.L] : c_half[td.L]) : 100.0);
+        c_max = std::max(c_max, c);
+        c_sum += c;
     }
-    if (ck > (size_t)optin) return fail(EA_EINVAL, "the colour-order sweep does not fit in shared memory");
-    *ck_smem_out = ck;
-    *parities = par;
-    return EA_OK;
+    const double n_sm = std::max(ctx->n_sm, 1), nt = (double)ctx->tiles.size();
+    const double t_walk = 23.0 * w_max + 10.2 * w_sum / (4.0 * n_sm);
+    const double t_checker = std::max(c_max, std::ceil(nt / n_sm) * c_sum / nt);
+    return have && t_checker < t_walk ? checker : walk;
 }
 
 // the context's sweeps in its order and launch configuration, queued on its stream (also the
@@ -659,15 +687,19 @@ int ctx_enqueue_sweeps(ea_ctx *ctx, uint64_t n_sweeps, int count_roundtrips) {
     const int nt = (int)ctx->tiles.size();
     const uint64_t chunk = ctx->sweeps_per_launch ? ctx->sweeps_per_launch : n_sweeps;
     if (ctx->order == 1) {
-        int rc, parities = 0;
-        size_t ck_smem = 0;
-        if ((rc = colour_launch(ctx, &ck_smem, &parities))) return rc;
+        const ColourPlan plan = colour_plan(ctx);
         unsigned *diag = reinterpret_cast<unsigned *>(ctx->d_queue + 1);
-        for (uint64_t done = 0; done < n_sweeps && ck_smem > 0; done += chunk) {
+        for (uint64_t done = 0; done < n_sweeps; done += chunk) {
             const uint64_t now = std::min(chunk, n_sweeps - done);
-            EA_CUDA(launch_sweeps_checker(ctx->d_tiles, nt, ctx->dim, ck_smem, ctx->d_slots, ctx->d_spins,
+            if (plan.walk) {
+                EA_CUDA(launch_sweeps_walk(ctx->d_tiles, ctx->d_order, nt, ctx->dim, plan.max_width, plan.smem,
+                                           ctx->d_slots, ctx->d_spins, ctx->d_bonds, ctx->d_thr, ctx->d_hist, now,
+                                           ctx->key, count_roundtrips, diag, ctx->stream));
+                continue;
+            }
+            EA_CUDA(launch_sweeps_checker(ctx->d_tiles, nt, ctx->dim, plan.smem, ctx->d_slots, ctx->d_spins,
                                           ctx->d_bonds, ctx->d_thr, ctx->d_hist, now, ctx->key, count_roundtrips,
-                                          diag, ctx->stream, parities));
+                                          diag, ctx->stream, plan.parities));
         }
         return EA_OK;
     }
@@ -735,7 +767,7 @@ extern "C" int muca_set_tile_width(ea_ctx *ctx, int L, int width) {
     if (!ctx) return fail(EA_EINVAL, "null context");
     if (L < 3 || L > 12) return fail(EA_EINVAL, "L must be in [3, 12] (got %d)", L);
     const int dim = ctx->dim ? ctx->dim : 3;
-    if (!sweep_width_supported(dim, L, width) && checker_smem_bytes(dim, L, width) == 0)
+    if (!sweep_width_supported(dim, L, width) && !colour_width_supported(dim, L, width))
         return fail(EA_EINVAL, "tile width %d is not available for dim=%d, L=%d (32 always; in 3D 16 for "
                                "L=7,8, and in the colour order 8 for L=9,10 and 4 for L=11,12)", width, dim, L);
     ctx->tile_width[L] = width;
@@ -750,10 +782,10 @@ extern "C" int muca_get_tile_width(int dim, int L, int width, size_t *smem_bytes
 }
 
 extern "C" int muca_get_tile_width_colour(int dim, int L, int width, size_t *smem_bytes, int *thresholds_in_smem) {
-    const size_t b = checker_smem_bytes(dim, L, width);
-    if (b == 0) return fail(EA_EINVAL, "tile width %d unavailable in the colour order", width);
-    if (smem_bytes) *smem_bytes = b;
-    if (thresholds_in_smem) *thresholds_in_smem = checker_thresholds_in_smem(dim, L, width) ? 1 : 0;
+    if (!colour_width_supported(dim, L, width))
+        return fail(EA_EINVAL, "tile width %d unavailable in the colour order", width);
+    if (smem_bytes) *smem_bytes = walk_smem_bytes(dim, L);
+    if (thresholds_in_smem) *thresholds_in_smem = 1;  // the part around the current bin
     return EA_OK;
 }
 

@@ -106,17 +106,24 @@ cudaError_t launch_sweeps(const TileDesc *d_tiles, const int32_t *d_tile_list, i
                           const uint32_t *d_bonds, const uint32_t *d_thr, uint32_t *d_hist, uint64_t n_sweeps,
                           PhiloxKey key, int count_rt, unsigned *d_diag, cudaStream_t st);
 int sweep_blocks_per_sm(int dim, size_t smem);
-// the colour-order sweep (muca_checker.cu): one lane per chain, every L; widths 32 and (3D) 16 at
-// L = 7, 8, 8 at L = 9, 10, 4 at L = 11, 12 (0 bytes: not available)
+// the colour-order sweep, one warp per chain (muca_walk.cu): every L and tile width; d_list: the tiles,
+// longest first
+bool colour_width_supported(int dim, int L, int width);
+size_t walk_smem_bytes(int dim, int L);
+cudaError_t launch_sweeps_walk(const TileDesc *d_tiles, const int32_t *d_list, int n_tiles, int dim, int max_width,
+                               size_t smem, SlotState *d_slots, uint32_t *d_spins, const uint32_t *d_bonds,
+                               const uint32_t *d_thr, uint32_t *d_hist, uint64_t n_sweeps, PhiloxKey key,
+                               int count_rt, unsigned *d_diag, cudaStream_t st);
+// the colour-order sweep, one lane per chain (muca_checker.cu): every L in full tiles, and 3D tiles of
+// 16 at L = 4..8 (0 bytes: not available)
 size_t checker_smem_bytes(int dim, int L, int width);
-bool checker_thresholds_in_smem(int dim, int L, int width);
-// the kernel-form class of a tile in the colour order: 1 even L, 2 odd L, 4 the narrow tiles of the
-// small even sizes (3D, L <= 6), which run in forms of their own
+// the kernel-form class of a tile there: 1 even L, 2 odd L, 4 the narrow tiles of the small even sizes
+// (3D, L <= 6), which run in forms of their own
 int checker_parity_class(int dim, int L, int width);
 cudaError_t launch_sweeps_checker(const TileDesc *d_tiles, int n_tiles, int dim, size_t smem, SlotState *d_slots,
                                   uint32_t *d_spins, const uint32_t *d_bonds, const uint32_t *d_thr,
                                   uint32_t *d_hist, uint64_t n_sweeps, PhiloxKey key, int count_rt,
-                                  unsigned *d_diag, cudaStream_t st, int parities);  // bit 0 even L, bit 1 odd L
+                                  unsigned *d_diag, cudaStream_t st, int parities);
 cudaError_t prepare_sweeps(int dim, size_t smem);  // resident sweep blocks per SM at this smem
 cudaError_t launch_quantize(const TileDesc *d_tiles, int n_tiles, const SlotState *d_slots,
                             const double *d_lnW, uint32_t *d_thr, cudaStream_t st);
