@@ -19,17 +19,30 @@
 // the 32 realizations' thresholds.  The comparison runs over planes from the most
 // significant one: the first 8 without branches, the rest only while a bit is undecided.
 //
+// What bounds it.  A site word costs two Philox calls (40 wide multiplies at a quarter of the issue
+// rate), about 40 operations of the comparison and 25 for its neighbours, most of them at half rate, so
+// a batch that fills the SMs (L = 8, 1024 x 32: two CTAs on two SMs of three) is bound by those pipes;
+// between the colour passes a CTA walks a chain of short steps (open comparisons, energies, exchange)
+// whose latencies add up: 13 of 29 thousand cycles a sweep before they were shortened, 7 now.
+// us per sweep, before -> now: 1024 x 32 of L = 8 15.9 -> 11.6 (1056 -> 1447 attempts/ns); 32 x 32 of
+// L = 8 11.3 -> 7.1; 1024 x 14 of L = 6 7.4 -> 5.3; 128 x 20 of L = 12 35 -> 23; 333 x 12 of L = 5 6.7 ->
+// 4.6; 256 x 17 of L = 7 36 -> 24.
+//
 // Parallel work.  One thread-block cluster per group: CS CTAs, each owning M/CS consecutive
-// slots in shared memory.  Energies are recomputed after every sweep (bit-sliced counters,
-// warp bit-matrix transpose, popcount); exchanges between slots owned by different CTAs read
-// and write the neighbour CTA's shared memory (distributed shared memory) between cluster
-// barriers.
+// slots in shared memory; a thread keeps its sites (index, neighbours, bonds) and goes through
+// the slots.  Energies come from the updates themselves (bit-sliced counts, warp bit-matrix
+// transpose, popcount): for even L the unsatisfied bonds counted at the second colour's sites, for
+// odd L the change at every site, instead of a pass over all bonds.  Exchanges between slots owned by
+// different CTAs read and write the neighbour CTA's shared memory (distributed shared memory)
+// between cluster barriers, all loads before the stores; a replica's round-trip record moves with it,
+// so that the check after the exchange is local.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "eamc.h"
@@ -71,16 +84,19 @@ __device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
     return (a & b) | (a & c) | (b & c);
 }
 
-// 32x32 bit-matrix transpose across a warp: afterwards lane t holds, in bit s, bit t of
-// what lane s held
+// 32x32 bit-matrix transpose across a warp: afterwards lane t holds, in bit s, bit t of what lane s
+// held.  Stage j swaps the off-diagonal j x j blocks: a lane keeps the bits of mask k, and takes the
+// others from its partner's word rotated by j (down where its own bit j is set): one shuffle, one
+// rotation, one three-input operation a stage
 __device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
     const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
 #pragma unroll
     for (int s = 0; s < 5; ++s) {
         const int j = 16 >> s;
-        const uint32_t m = masks[s];
+        const uint32_t keep = (lane & j) ? ~masks[s] : masks[s];
         const uint32_t y = __shfl_xor_sync(kFull, x, j);
-        x = (lane & j) ? ((x & ~m) | ((y & ~m) >> j)) : ((x & m) | ((y & m) << j));
+        const uint32_t r = __funnelshift_l(y, y, (lane & j) ? 32 - j : j);
+        x = (x & keep) | (r & ~keep);
     }
     return x;
 }
@@ -90,7 +106,36 @@ struct PtGeo {
     static constexpr int NR = DIM == 3 ? L * L : L;
     static constexpr int V = NR * L;
     static constexpr int NB = DIM * V;
-    static constexpr int HALF = V / 2;  // sites of one colour
+    static constexpr int HALF = V / 2;  // sites of one colour (even L)
+    static constexpr bool ODD = (L & 1) != 0;
+    // most sites of one colour, odd L: the axis colours 0, 1, 2 of L positions occur n0, n1, n2 times;
+    // the fullest class of their DIM-fold sums mod 3
+    static constexpr int axn(int c) {
+        int n = 0;
+        for (int x = 0; x < L; ++x) n += ((x == L - 1 && (L - 1) % 3 == 0) ? 1 : x % 3) == c;
+        return n;
+    }
+    static constexpr int most_odd() {
+        int best = 0;
+        for (int c = 0; c < 3; ++c) {
+            int n = 0;
+            for (int a = 0; a < 3; ++a)
+                for (int b = 0; b < 3; ++b) {
+                    if (DIM == 3) n += axn(a) * axn(b) * axn(((c - a - b) % 3 + 3) % 3);
+                    else if ((a + b) % 3 == c) n += axn(a) * axn(b);
+                }
+            best = n > best ? n : best;
+        }
+        return best;
+    }
+    static constexpr int NC = ODD ? most_odd() : HALF;
+    // a block's threads: JT over the sites of a colour (whole warps, in NP passes where the sites are more
+    // than 288), times KT slots side by side
+    static constexpr int NP = (NC + 287) / 288;
+    static constexpr int JT = ((NC + NP - 1) / NP + 31) / 32 * 32;
+    static constexpr int KT_MAX = JT > 128 ? 1 : 256 / JT;
+    static __host__ __device__ constexpr int kt(int spc) { return spc < KT_MAX ? spc : KT_MAX; }
+    static __host__ __device__ constexpr int threads(int spc) { return JT * kt(spc); }
 };
 
 // neighbour of site i along axis d (0 x, 1 y, 2 z), direction +1 / -1
@@ -145,9 +190,10 @@ struct PtArgs {
 };
 
 template <int DIM, int L>
-__global__ void __launch_bounds__(256, 1) pt_kernel(PtArgs a) {
+__global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
     using G = PtGeo<DIM, L>;
     constexpr int V = G::V, NB = G::NB, HALF = G::HALF;
+    constexpr bool ODD = G::ODD;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int g = blockIdx.x / (int)cluster.num_blocks();
@@ -169,11 +215,11 @@ __global__ void __launch_bounds__(256, 1) pt_kernel(PtArgs a) {
     uint32_t *Xc = (uint32_t *)(Ep + nwarps * spc * 32);  // [spc][32] accepted exchanges, this launch
     int32_t *Bd = (int32_t *)(Xc + spc * 32);             // [32][2] round-trip bounds (e_g, e_hot)
     double *Db = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(Bd + 64) + 7) & ~uintptr_t(7));  // [spc][32]
-    // round-trip records of the replica labels k0 .. k0+spc-1 ("home" labels of this CTA), for
-    // the launch; a label's record is updated by whichever CTA holds that replica, through
-    // distributed shared memory
+    // round-trip records of the replicas in the CTA's slots, for the launch; an exchange moves them with
+    // the configurations
     PtRt *Rh = reinterpret_cast<PtRt *>(Db + spc * 32);    // [spc][32]
-    int32_t *Cl = (int32_t *)(Rh + spc * 32);  // odd L: sites by colour [V], then offsets [4]
+    float *Df = reinterpret_cast<float *>(Rh + spc * 32);  // [spc][32] Db in single precision
+    int32_t *Cl = (int32_t *)(Df + spc * 32);  // odd L: sites by colour [V], then offsets [4]
 
     const uint32_t group_rid0 = a.rid0 + 32u * (uint32_t)g;
     const int nvalid = min(32, a.n_real - 32 * g);
@@ -184,7 +230,9 @@ __global__ void __launch_bounds__(256, 1) pt_kernel(PtArgs a) {
     for (int k = tid; k < NB; k += blockDim.x) J[k] = a.bonds[(size_t)g * NB + k];
     for (int k = tid; k < spc * 32; k += blockDim.x) {
         Es[k] = a.E[((size_t)g * M + k0) * 32 + k];
-        Ls[k] = a.label[((size_t)g * M + k0) * 32 + k];
+        const int label = a.label[((size_t)g * M + k0) * 32 + k];
+        Ls[k] = label;
+        Rh[k] = a.rt[((size_t)g * M + label) * 32 + (k & 31)];
     }
     for (int k = tid; k < spc * 128; k += blockDim.x) sm[k] = a.planes[((size_t)g * M + k0) * 128 + k];
     // per launch: beta_{k+1} - beta_k of every owned pair and realization, the round-trip bounds,
@@ -192,10 +240,10 @@ __global__ void __launch_bounds__(256, 1) pt_kernel(PtArgs a) {
     for (int q = tid; q < spc * 32; q += blockDim.x) {
         const int k = k0 + (q >> 5), b = q & 31;
         Db[q] = (k + 1 < M) ? a.beta[((size_t)g * M + k + 1) * 32 + b] - a.beta[((size_t)g * M + k) * 32 + b] : 0.0;
+        Df[q] = (float)Db[q];
         Xc[q] = 0u;
     }
     for (int q = tid; q < 64; q += blockDim.x) Bd[q] = a.bounds[(size_t)g * 64 + q];
-    for (int q = tid; q < spc * 32; q += blockDim.x) Rh[q] = a.rt[((size_t)g * M + k0) * 32 + q];
     if constexpr ((L & 1) != 0) {
         if (tid == 0) {  // colour classes in lexicographic order (a few thousand steps per launch)
             int n = 0;
@@ -210,116 +258,163 @@ __global__ void __launch_bounds__(256, 1) pt_kernel(PtArgs a) {
     __syncthreads();
     cluster.sync();
 
+    // this thread's sites of a colour are jt, jt + JT, ..., its slots kt, kt + KT, ...
+    const int KT = G::kt(spc), jt = tid % G::JT, kt = tid / G::JT;
+    const int nk = (spc + KT - 1) / KT;
     for (uint64_t s = 0; s < a.n_sweeps; ++s) {
         const uint64_t t = a.t0 + s;
         const uint32_t tt = (uint32_t)t;
         // ---- checkerboard Metropolis sweep of every owned slot
-        // planes 8..31 of one site word: drawn only while a bit is still undecided
+        // planes 8..31 of one site word: 8..15 together (two calls side by side decide all but about
+        // 2^-8 of the words that come here), the rest while a bit is still undecided
         auto finish = [&](int i, int ks, uint32_t C0, uint32_t C1, uint32_t C2, uint32_t acc, uint32_t und) {
             const uint32_t c2 = (uint32_t)g + (a.rid0 >> 5), c3 = 4u | ((uint32_t)(k0 + ks) << 8);
             const uint4 *Pk = P + ks * 32;
-            uint4 w4 = make_uint4(0, 0, 0, 0);
-            for (int m = 8; m < 32 && und; ++m) {
-                if ((m & 3) == 0)
-                    w4 = philox4x32_10(make_uint4((uint32_t)(8 * i + (m >> 2)), tt, c2, c3), a.key);
-                const uint32_t R = uint4_get(w4, m & 3);
-                const uint4 q = Pk[m];
-                const uint32_t Tm = (C0 & q.x) | (C1 & q.y) | (C2 & q.z);
-                acc |= und & ~R & Tm;
-                und &= ~(R ^ Tm);
-            }
+            auto planes = [&](const uint4 &w, int m0) {
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const uint32_t R = uint4_get(w, m);
+                    const uint4 q = Pk[m0 + m];
+                    const uint32_t Tm = (C0 & q.x) | (C1 & q.y) | (C2 & q.z);
+                    acc |= und & ~R & Tm;
+                    und &= ~(R ^ Tm);
+                }
+            };
+            const uint4 wa = philox4x32_10(make_uint4((uint32_t)(8 * i + 2), tt, c2, c3), a.key);
+            const uint4 wb = philox4x32_10(make_uint4((uint32_t)(8 * i + 3), tt, c2, c3), a.key);
+            planes(wa, 8);
+            planes(wb, 12);
+#pragma unroll 1
+            for (int m = 16; m < 32 && und; m += 4)
+                planes(philox4x32_10(make_uint4((uint32_t)(8 * i + (m >> 2)), tt, c2, c3), a.key), m);
             return acc;
         };
         uint32_t *tq = TQ + warp * kTailQ * 6;
         for (int colour = 0; colour < NCOL; ++colour) {
-            const int nc = ((L & 1) == 0) ? HALF : Cl[V + colour + 1] - Cl[V + colour];
+            const int nc = ODD ? Cl[V + colour + 1] - Cl[V + colour] : HALF;
             // site words of one colour never neighbour each other, so a word whose comparison
             // is still open after 8 planes (about 6 % of them) can be finished after the others:
             // the warp queues them and finishes them together, one per lane
             int nq = 0;
-            for (int item = tid; item < spc * nc; item += blockDim.x) {
-                const int ks = item / nc, j = item % nc;
-                int i;
-                if constexpr ((L & 1) == 0) {
-                    const int row = j / (L / 2), xh = j % (L / 2);
+            for (int pass = 0; pass < G::NP; ++pass) {
+                const int j = jt + pass * G::JT;
+                const bool site = j < nc;
+                // the site, its neighbours and its bonds: the same for every slot
+                int i = 0;
+                if constexpr (!ODD) {
+                    const int row = site ? j / (L / 2) : 0, xh = site ? j % (L / 2) : 0;
                     const int y = row % L, z = DIM == 3 ? row / L : 0;
                     i = 2 * xh + ((colour + y + z) & 1) + L * row;
                 } else {
-                    i = Cl[Cl[V + colour] + j];
+                    if (site) i = Cl[Cl[V + colour] + j];
                 }
-                uint32_t *Sk = S + ks * V;
-                const uint32_t si = Sk[i];
-                uint32_t u[2 * DIM];
+                int nb[2 * DIM];
+                uint32_t jw[2 * DIM];
 #pragma unroll
                 for (int d = 0; d < DIM; ++d) {
-                    const int jp = pt_nbr<DIM, L>(i, d, +1), jm = pt_nbr<DIM, L>(i, d, -1);
-                    u[2 * d] = si ^ Sk[jp] ^ J[i * DIM + d];
-                    u[2 * d + 1] = si ^ Sk[jm] ^ J[jm * DIM + d];
+                    nb[2 * d] = pt_nbr<DIM, L>(i, d, +1);
+                    nb[2 * d + 1] = pt_nbr<DIM, L>(i, d, -1);
+                    jw[2 * d] = J[i * DIM + d];
+                    jw[2 * d + 1] = J[nb[2 * d + 1] * DIM + d];
                 }
-                uint32_t n0, n1, n2;  // bit-sliced count of unsatisfied bonds
-                if constexpr (DIM == 3) {
-                    const uint32_t s1 = u[0] ^ u[1] ^ u[2], c1 = maj3(u[0], u[1], u[2]);
-                    const uint32_t s2 = u[3] ^ u[4] ^ u[5], c2 = maj3(u[3], u[4], u[5]);
-                    n0 = s1 ^ s2;
-                    const uint32_t c3 = s1 & s2;
-                    n1 = c1 ^ c2 ^ c3;
-                    n2 = maj3(c1, c2, c3);
-                } else {
-                    const uint32_t s1 = u[0] ^ u[1] ^ u[2], c1 = maj3(u[0], u[1], u[2]);
-                    n0 = s1 ^ u[3];
-                    const uint32_t c2 = s1 & u[3];
-                    n1 = c1 ^ c2;
-                    n2 = c1 & c2;
-                }
-                // uphill classes: n < DIM unsatisfied bonds (dE = 2*(2*DIM) - 4n > 0)
-                uint32_t C[3];
-                C[0] = ~n2 & ~n1 & ~n0;
-                C[1] = ~n2 & ~n1 & n0;
-                C[2] = (DIM == 3) ? (~n2 & n1 & ~n0) : 0u;
-                const uint32_t up = C[0] | C[1] | C[2];
-                uint32_t acc = ~up;  // dE <= 0 always accepted
-                uint32_t und = up & valid;
-                const int k = k0 + ks;
-                const uint4 *Pk = P + ks * 32;
-                // the 8 most significant planes come from two independent Philox calls and are
-                // compared without branches; planes 8..31 are drawn only while a bit is still
-                // undecided (about 2^-8 per uphill bit)
-                const uint32_t c2 = (uint32_t)g + (a.rid0 >> 5), c3 = 4u | ((uint32_t)k << 8);
-                const uint4 wa = philox4x32_10(make_uint4((uint32_t)(8 * i), tt, c2, c3), a.key);
-                const uint4 wb = philox4x32_10(make_uint4((uint32_t)(8 * i + 1), tt, c2, c3), a.key);
-                const uint32_t Rm[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+                const uint32_t c2 = (uint32_t)g + (a.rid0 >> 5);
+                for (int it = 0; it < nk; ++it) {
+                    const int ks = kt + it * KT;
+                    const bool act = site && ks < spc;
+                    uint32_t *Sk = S + (act ? ks : 0) * V;
+                    const uint32_t si = Sk[i];
+                    uint32_t u[2 * DIM];
 #pragma unroll
-                for (int m = 0; m < 8; ++m) {
-                    const uint4 q = Pk[m];
-                    const uint32_t Tm = (C[0] & q.x) | (C[1] & q.y) | (C[2] & q.z);
-                    acc |= und & ~Rm[m] & Tm;  // r bit 0, threshold bit 1: r < threshold
-                    und &= ~(Rm[m] ^ Tm);      // equal bits: still undecided
+                    for (int d = 0; d < 2 * DIM; ++d) u[d] = si ^ Sk[nb[d]] ^ jw[d];
+                    uint32_t n0, n1, n2;  // bit-sliced count of unsatisfied bonds
+                    if constexpr (DIM == 3) {
+                        const uint32_t s1 = u[0] ^ u[1] ^ u[2], c1 = maj3(u[0], u[1], u[2]);
+                        const uint32_t s2 = u[3] ^ u[4] ^ u[5], d1 = maj3(u[3], u[4], u[5]);
+                        n0 = s1 ^ s2;
+                        const uint32_t c3 = s1 & s2;
+                        n1 = c1 ^ d1 ^ c3;
+                        n2 = maj3(c1, d1, c3);
+                    } else {
+                        const uint32_t s1 = u[0] ^ u[1] ^ u[2], c1 = maj3(u[0], u[1], u[2]);
+                        n0 = s1 ^ u[3];
+                        const uint32_t d1 = s1 & u[3];
+                        n1 = c1 ^ d1;
+                        n2 = c1 & d1;
+                    }
+                    // uphill classes: n < DIM unsatisfied bonds (dE = 2*(2*DIM) - 4n > 0)
+                    uint32_t C[3];
+                    C[0] = ~n2 & ~n1 & ~n0;
+                    C[1] = ~n2 & ~n1 & n0;
+                    C[2] = (DIM == 3) ? (~n2 & n1 & ~n0) : 0u;
+                    const uint32_t up = C[0] | C[1] | C[2];
+                    uint32_t acc = ~up;  // dE <= 0 always accepted
+                    uint32_t und = act ? up & valid : 0u;
+                    const uint4 *Pk = P + (act ? ks : 0) * 32;
+                    // the 8 most significant planes come from two independent Philox calls and are
+                    // compared without branches; planes 8..31 are drawn only while a bit is still
+                    // undecided (about 2^-8 per uphill bit)
+                    const uint32_t c3 = 4u | ((uint32_t)(k0 + ks) << 8);
+                    const uint4 wa = philox4x32_10(make_uint4((uint32_t)(8 * i), tt, c2, c3), a.key);
+                    const uint4 wb = philox4x32_10(make_uint4((uint32_t)(8 * i + 1), tt, c2, c3), a.key);
+                    const uint32_t Rm[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+                    // from the least significant of the eight: less = (r < threshold) on the bits so far, one
+                    // three-input operation a plane (below: r bit 0, threshold bit 1; equal: as before)
+                    uint32_t less = 0u, same = und;
+#pragma unroll
+                    for (int m = 7; m >= 0; --m) {
+                        const uint4 q = Pk[m];
+                        const uint32_t Tm = (C[0] & q.x) | (C[1] & q.y) | (C[2] & q.z);
+                        less = (~Rm[m] & Tm) | (~(Rm[m] ^ Tm) & less);
+                        same &= ~(Rm[m] ^ Tm);
+                    }
+                    acc |= und & less;
+                    und = same;
+                    const bool open = und != 0u;
+                    const uint32_t om = __ballot_sync(kFull, open);
+                    const int pos = nq + __popc(om & ((1u << lane) - 1u));
+                    const bool deferred = open && pos < kTailQ;
+                    if (deferred) {
+                        uint32_t *e = tq + pos * 6;
+                        e[0] = (uint32_t)i | ((uint32_t)ks << 16);
+                        e[1] = acc;
+                        e[2] = und;
+                        e[3] = C[0];
+                        e[4] = C[1];
+                        e[5] = C[2];
+                    } else if (act) {
+                        if (open) acc = finish(i, ks, C[0], C[1], C[2], acc, und);  // queue full
+                        Sk[i] = si ^ (acc & valid);
+                    }
+                    nq += __popc(om);
+                    // the slot's energy from the updates.  Even L: every bond has one end of the second
+                    // colour, so the unsatisfied bonds are the sum of n over its sites, after the update
+                    // (2 DIM - n where the spin flipped).  Odd L: the sum over all sites of 2 DIM - n where it
+                    // flipped and DIM where not, the change against all DIM.  A deferred word counts with the
+                    // bits decided so far.
+                    if (ODD || colour == 1) {
+                        const uint32_t in = act ? kFull : 0u, f = acc & valid & in;
+                        const uint32_t r0 = n0, r1 = DIM == 3 ? n1 ^ ~n0 : n1 ^ n0;  // 2 DIM - n
+                        const uint32_t r2 = DIM == 3 ? ~n2 & ~(n1 & n0) : ~n2 & ~n1 & ~n0;
+                        uint32_t m0, m1, m2;
+                        if constexpr (ODD) {
+                            m0 = (f & r0) | (DIM == 3 ? ~f : 0u);
+                            m1 = (f & r1) | ~f;
+                            m2 = f & r2;
+                        } else {
+                            m0 = n0;
+                            m1 = (f & r1) | (~f & n1);
+                            m2 = (f & r2) | (~f & n2);
+                        }
+                        const int part = __popc(warp_transpose(m0 & in, lane)) + 2 * __popc(warp_transpose(m1 & in, lane)) +
+                                         4 * __popc(warp_transpose(m2 & in, lane));
+                        if (ks < spc) {
+                            int32_t *e = Ep + ((jt >> 5) * spc + ks) * 32 + lane;
+                            *e = (pass == 0 && (!ODD || colour == 0)) ? part : *e + part;
+                        }
+                    }
                 }
-                (void)c2;
-                (void)c3;
-                // the lanes of this warp that have an item in this pass of the loop (items are consecutive)
-                const int rem = spc * nc - (item - lane);
-                const uint32_t live = rem >= 32 ? kFull : ((1u << rem) - 1u);
-                const bool open = und != 0u;
-                const uint32_t om = __ballot_sync(live, open);
-                const int pos = nq + __popc(om & ((1u << lane) - 1u));
-                const bool deferred = open && pos < kTailQ;
-                if (deferred) {
-                    uint32_t *e = tq + pos * 6;
-                    e[0] = (uint32_t)i | ((uint32_t)ks << 16);
-                    e[1] = acc;
-                    e[2] = und;
-                    e[3] = C[0];
-                    e[4] = C[1];
-                    e[5] = C[2];
-                } else {
-                    if (open) acc = finish(i, ks, C[0], C[1], C[2], acc, und);  // queue full
-                    Sk[i] = si ^ (acc & valid);
-                }
-                nq += __popc(om);
             }
             __syncwarp();
-            nq = __shfl_sync(kFull, nq, 0);
             for (int e0 = 0; e0 < min(nq, kTailQ); e0 += 32) {
                 const int e = e0 + lane;
                 if (e < min(nq, kTailQ)) {
@@ -327,96 +422,125 @@ __global__ void __launch_bounds__(256, 1) pt_kernel(PtArgs a) {
                     const int i = (int)(q[0] & 0xFFFFu), ks = (int)(q[0] >> 16);
                     const uint32_t acc = finish(i, ks, q[3], q[4], q[5], q[1], q[2]);
                     S[ks * V + i] ^= acc & valid;
+                    if (ODD || colour == 1) {  // bits accepted only now
+                        uint32_t late = acc & ~q[1] & valid;
+                        while (late) {
+                            const int b = __ffs(late) - 1;
+                            late &= late - 1u;
+                            const int n = (int)((q[4] >> b) & 1u) + 2 * (int)((q[5] >> b) & 1u);
+                            atomicAdd(&Ep[((jt >> 5) * spc + ks) * 32 + b], ODD ? DIM - n : 2 * DIM - 2 * n);
+                        }
+                    }
                 }
             }
             __syncthreads();
         }
-        // ---- energies of the owned slots: u_b = number of unsatisfied bonds of bit b; every
-        //      warp leaves its partial counts in Ep, one barrier, then they are summed
-        for (int ks = 0; ks < spc; ++ks) {
-            const uint32_t *Sk = S + ks * V;
-            int part = 0;
-            for (int base = warp * 32; base < V; base += nwarps * 32) {
-                const int i = base + lane;
-                uint32_t c0 = 0, c1 = 0;  // bit-sliced count (0..3) of this site's +d bonds
-                if (i < V) {
-#pragma unroll
-                    for (int d = 0; d < DIM; ++d) {
-                        const uint32_t w = Sk[i] ^ Sk[pt_nbr<DIM, L>(i, d, +1)] ^ J[i * DIM + d];
-                        c1 ^= c0 & w;  // add one bit into the 2-bit counter (max 3)
-                        c0 ^= w;
-                    }
-                }
-                const uint32_t t0w = warp_transpose(c0, lane), t1w = warp_transpose(c1, lane);
-                part += __popc(t0w) + 2 * __popc(t1w);
-            }
-            Ep[(warp * spc + ks) * 32 + lane] = part;
-        }
-        __syncthreads();
+        // ---- energies of the owned slots from the warps' sums
         for (int k = tid; k < spc * 32; k += blockDim.x) {
             int u = 0;
-            for (int w = 0; w < nwarps; ++w) u += Ep[w * spc * 32 + k];
-            Es[k] = 2 * u - NB;
+#pragma unroll
+            for (int w = 0; w < G::JT / 32; ++w) u += Ep[w * spc * 32 + k];
+            Es[k] = ODD ? Es[k] + 4 * (u - DIM * V) : 2 * u - NB;
         }
         cluster.sync();  // every slot's energy is known (and a barrier of this CTA)
         // ---- replica exchange between (k, k+1), k = t mod 2 (mod 2); the owner of k decides,
-        //      one warp per owned slot
-        {
-            for (int ks = warp; ks < spc; ks += nwarps) {
-                const int k = k0 + ks;
-                uint32_t A = 0u;
-                if (((k ^ (int)t) & 1) == 0 && k + 1 < M) {
-                    const int kr = (ks + 1 < spc) ? rank : rank + 1;
-                    const int ksr = (ks + 1 < spc) ? ks + 1 : 0;
-                    int32_t *Er = cluster.map_shared_rank(Es, kr);
-                    const int e0 = Es[ks * 32 + lane], e1 = Er[ksr * 32 + lane];
-                    bool ok;
-                    if (e1 >= e0) {
-                        ok = true;
-                    } else {
-                        // Eq. "temperatureexchange" with this realization's beta_k, beta_k+1
-                        const int d = (e0 - e1) / 4;
-                        const uint32_t th = quantize_prob(exp(-Db[ks * 32 + lane] * 4.0 * (double)d));
-                        const uint4 w = philox4x32_10(make_uint4((uint32_t)k, tt, group_rid0 + lane, 1u), a.key);
-                        ok = (th == kAlways) || (w.x < th);
-                    }
-                    A = __ballot_sync(kFull, ok) & valid;
-                    Xc[ks * 32 + lane] += (A >> lane) & 1u;
-                }
-                if (lane == 0) Amask[ks] = A;
-            }
-        }
-        __syncthreads();
-        for (int ks = 0; ks < spc; ++ks) {
-            const uint32_t A = Amask[ks];
-            if (!A) continue;  // uniform across the CTA
+        //      one warp per owned pair ks0, ks0 + 2, ...
+        const int ks0 = (k0 ^ (int)t) & 1;
+        const int np = max(0, (min(spc, M - 1 - k0) - ks0 + 1) / 2);
+        for (int p = warp; p < np; p += nwarps) {
+            const int ks = ks0 + 2 * p, k = k0 + ks;
             const int kr = (ks + 1 < spc) ? rank : rank + 1;
             const int ksr = (ks + 1 < spc) ? ks + 1 : 0;
-            uint32_t *Sr = cluster.map_shared_rank(S, kr) + ksr * V;
-            uint32_t *Sl = S + ks * V;
-            for (int i = tid; i < V; i += blockDim.x) {
-                const uint32_t d = (Sl[i] ^ Sr[i]) & A;
-                Sl[i] ^= d;
-                Sr[i] ^= d;
+            const int32_t *Er = cluster.map_shared_rank(Es, kr);
+            const int e0 = Es[ks * 32 + lane], e1 = Er[ksr * 32 + lane];
+            const uint4 w = philox4x32_10(make_uint4((uint32_t)k, tt, group_rid0 + lane, 1u), a.key);
+            bool ok = true;
+            if (e1 < e0) {
+                // Eq. "temperatureexchange" with this realization's beta_k, beta_k+1: accepted with
+                // p = exp(-x), quantised to 32 bits.  In single precision p is known to 1e-5; the exact
+                // threshold (FP64, 32 times slower) is needed only where the word lies that close to it
+                const int d4 = (e0 - e1) / 4;
+                const float x = Df[ks * 32 + lane] * (4.0f * (float)d4), pf = expf(-x) * 4294967296.0f, wf = (float)w.x;
+                const float slack = (2e-6f + 1e-6f * x) * pf + 1e-6f * wf + 4.0f;
+                ok = wf < pf;
+                if (!(fabsf(wf - pf) > slack)) {
+                    const uint32_t th = quantize_prob(exp(-Db[ks * 32 + lane] * 4.0 * (double)d4));
+                    ok = (th == kAlways) || (w.x < th);
+                }
             }
-            if (tid < 32 && ((A >> tid) & 1u)) {
-                int32_t *Er = cluster.map_shared_rank(Es, kr);
-                int32_t *Lr = cluster.map_shared_rank(Ls, kr);
-                const int32_t te = Es[ks * 32 + tid];
-                Es[ks * 32 + tid] = Er[ksr * 32 + tid];
-                Er[ksr * 32 + tid] = te;
-                const int32_t tl = Ls[ks * 32 + tid];
-                Ls[ks * 32 + tid] = Lr[ksr * 32 + tid];
-                Lr[ksr * 32 + tid] = tl;
+            const uint32_t A = __ballot_sync(kFull, ok) & valid;
+            Xc[ks * 32 + lane] += (A >> lane) & 1u;
+            if (lane == 0) Amask[ks] = A;
+        }
+        __syncthreads();
+        // the configurations, energies, labels and records of the accepted pairs change places; the pairs
+        // are disjoint, and all loads of a round (the neighbour CTA's shared memory) come before its stores
+        {
+            constexpr int VQ = (V % 4 == 0) ? 4 : 1;  // words per access
+            constexpr int Q = V / VQ;
+            using W = typename std::conditional<VQ == 4, uint4, uint32_t>::type;
+            const int ne = np * 32, nw = np * Q;
+            for (int e = tid; e < max(nw, ne); e += blockDim.x) {
+                W a0, b0, *pa = nullptr, *pb = nullptr;
+                uint32_t A = 0u;
+                if (e < nw) {
+                    const int ks = ks0 + 2 * (e / Q), i = e % Q;
+                    A = Amask[ks];
+                    if (A) {
+                        const bool far = ks + 1 >= spc;
+                        pa = reinterpret_cast<W *>(S + ks * V) + i;
+                        pb = reinterpret_cast<W *>(far ? cluster.map_shared_rank(S, rank + 1) : S + (ks + 1) * V) + i;
+                        a0 = *pa;
+                        b0 = *pb;
+                    }
+                }
+                bool moves = false;
+                int q0 = 0, q1 = 0, kr = rank;
+                int32_t ea = 0, eb = 0, la = 0, lb = 0;
+                PtRt ra, rb;
+                if (e < ne) {
+                    const int ks = ks0 + 2 * (e >> 5), bit = e & 31;
+                    moves = ((Amask[ks] >> bit) & 1u) != 0u;
+                    if (moves) {
+                        kr = (ks + 1 < spc) ? rank : rank + 1;
+                        q0 = ks * 32 + bit;
+                        q1 = ((ks + 1 < spc) ? ks + 1 : 0) * 32 + bit;
+                        ea = Es[q0];
+                        la = Ls[q0];
+                        ra = Rh[q0];
+                        eb = cluster.map_shared_rank(Es, kr)[q1];
+                        lb = cluster.map_shared_rank(Ls, kr)[q1];
+                        rb = cluster.map_shared_rank(Rh, kr)[q1];
+                    }
+                }
+                if (A) {
+                    if constexpr (VQ == 4) {
+                        const uint4 d = make_uint4((a0.x ^ b0.x) & A, (a0.y ^ b0.y) & A, (a0.z ^ b0.z) & A, (a0.w ^ b0.w) & A);
+                        *pa = make_uint4(a0.x ^ d.x, a0.y ^ d.y, a0.z ^ d.z, a0.w ^ d.w);
+                        *pb = make_uint4(b0.x ^ d.x, b0.y ^ d.y, b0.z ^ d.z, b0.w ^ d.w);
+                    } else {
+                        const uint32_t d = (a0 ^ b0) & A;
+                        *pa = a0 ^ d;
+                        *pb = b0 ^ d;
+                    }
+                }
+                if (moves) {
+                    Es[q0] = eb;
+                    Ls[q0] = lb;
+                    Rh[q0] = rb;
+                    cluster.map_shared_rank(Es, kr)[q1] = ea;
+                    cluster.map_shared_rank(Ls, kr)[q1] = la;
+                    cluster.map_shared_rank(Rh, kr)[q1] = ra;
+                }
             }
         }
         cluster.sync();  // exchanges complete everywhere
-        // ---- round trips / lowest energy per replica (by label)
+        // ---- round trips / lowest energy per replica; its record travels with it
         for (int q = tid; q < spc * 32; q += blockDim.x) {
-            const int ks = q >> 5, b = q & 31;
+            const int b = q & 31;
             if (!((valid >> b) & 1u)) continue;
-            const int lbl = Ls[q], E = Es[q];
-            PtRt &r = cluster.map_shared_rank(Rh, lbl / spc)[(lbl % spc) * 32 + b];
+            const int E = Es[q];
+            PtRt &r = Rh[q];
             if (E < r.e_min) r.e_min = E;
             if (a.count_rt) {
                 const int eg = Bd[2 * b + 0];
@@ -429,13 +553,12 @@ __global__ void __launch_bounds__(256, 1) pt_kernel(PtArgs a) {
                     if (E >= ehot) { r.n_rt += 1; r.t_last = (int64_t)t; r.phase = 1; }
                 }
             }
-            (void)ks;
         }
-        __syncthreads();
+        // (the next sweep writes energies, labels and records only after further barriers)
     }
-    // ---- write back (every CTA of the cluster is done with this CTA's records)
-    cluster.sync();
-    for (int q = tid; q < spc * 32; q += blockDim.x) a.rt[((size_t)g * M + k0) * 32 + q] = Rh[q];
+    __syncthreads();
+    // ---- write back; a replica's record to its label
+    for (int q = tid; q < spc * 32; q += blockDim.x) a.rt[((size_t)g * M + Ls[q]) * 32 + (q & 31)] = Rh[q];
     for (int q = tid; q < spc * 32; q += blockDim.x) {
         const int k = k0 + (q >> 5);
         if (Xc[q]) {
@@ -539,11 +662,10 @@ cudaError_t pt_launch_all(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, u
     a.n_sweeps = n_sweeps;
     a.count_rt = count_rt;
     a.key = ctx->key;
-    const int items = a.spc * (G::V / 2);
-    const int threads = std::min(256, std::max(64, (items + 31) / 32 * 32));
+    const int threads = G::threads(a.spc);
     const size_t smem = (size_t)(a.spc * 128 + a.spc * G::V + G::NB + a.spc * 32 * 2 + a.spc +
                                  (threads / 32) * (kTailQ * 6 + a.spc * 32) + a.spc * 32 + 64 + 1 + 2 * a.spc * 32 +
-                                 a.spc * 32 * (int)(sizeof(PtRt) / 4) + ((L & 1) ? G::V + 4 : 0)) * 4;
+                                 a.spc * 32 * (int)(sizeof(PtRt) / 4) + a.spc * 32 + ((L & 1) ? G::V + 4 : 0)) * 4;
     cudaError_t e = cudaFuncSetAttribute(pt_kernel<DIM, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(pt_kernel<DIM, L>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -551,8 +673,6 @@ cudaError_t pt_launch_all(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, u
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3(p->n_groups * p->cs);
-    // up to one thread per site of one colour of the CTA's slots (at most 256, at least 2
-    // warps); 512-thread blocks measured slower (barrier cost, register cap)
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = ctx->stream;
