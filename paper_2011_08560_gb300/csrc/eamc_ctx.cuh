@@ -18,6 +18,8 @@ struct ea_ctx {
     int max_V = 0;
     size_t sweep_smem = 0;    // dynamic shared memory of the sweep launch (largest tile)
     uint64_t max_t_host = 0;  // upper bound of every chain's sweep counter
+    bool thr_injected = false;  // some chain's thresholds may not be its weights' (muca_set_thresholds,
+                                // a snapshot): the next re-quantisation takes every chain
 
     // host mirrors
     std::vector<eamc::TileDesc> tiles;

@@ -127,6 +127,8 @@ cudaError_t launch_sweeps_checker(const TileDesc *d_tiles, int n_tiles, int dim,
 cudaError_t prepare_sweeps(int dim, size_t smem);  // resident sweep blocks per SM at this smem
 cudaError_t launch_quantize(const TileDesc *d_tiles, int n_tiles, const SlotState *d_slots,
                             const double *d_lnW, uint32_t *d_thr, cudaStream_t st);
+cudaError_t launch_quantize_selected(const TileDesc *d_tiles, int n_tiles, const SlotState *d_slots,
+                                     const double *d_lnW, uint32_t *d_thr, const uint8_t *d_sel, cudaStream_t st);
 cudaError_t launch_enforce_walls(const TileDesc *d_tiles, int n_tiles, const SlotState *d_slots,
                                  uint32_t *d_thr, cudaStream_t st);
 cudaError_t launch_update_weights(const TileDesc *d_tiles, int n_tiles, SlotState *d_slots,
