@@ -45,10 +45,21 @@ class ea_chain_desc(ctypes.Structure):
                 ("t", ctypes.c_uint64)]
 
 
+DESC_DTYPE = np.dtype([("dim", np.int32), ("L", np.int32), ("b_top", np.int32), ("parity", np.int32),
+                       ("rid", np.uint32), ("stream", np.uint32), ("E", np.int32), ("kind", np.int32),
+                       ("t", np.uint64)])
+assert DESC_DTYPE.itemsize == ctypes.sizeof(ea_chain_desc)
+
+
 class ea_pt_stats(ctypes.Structure):
     _fields_ = [("n_rt", ctypes.c_int32), ("phase", ctypes.c_int32),
                 ("t_first", ctypes.c_int64), ("t_last", ctypes.c_int64),
                 ("e_min", ctypes.c_int32), ("pad", ctypes.c_int32)]
+
+
+PT_DTYPE = np.dtype([(f, np.int64 if t is ctypes.c_int64 else np.int32) for f, t in ea_pt_stats._fields_])
+assert PT_DTYPE.itemsize == ctypes.sizeof(ea_pt_stats)
+assert RT_DTYPE.names[-1] == PT_DTYPE.names[-1] == "pad"
 
 
 class ea_srv_config(ctypes.Structure):
@@ -251,11 +262,17 @@ class Context:
     def num_chains(self) -> int:
         return lib().ea_num_chains(self._h)
 
+    def _describe(self, chain0: int, n: int) -> np.ndarray:
+        """Descriptions as a structured array: what the calls below need of them without a dict per
+        chain (12288 chains: 30 ms of Python)."""
+        out = np.zeros(max(n, 0), dtype=DESC_DTYPE)
+        check(lib().ea_describe(self._h, chain0, n, _p(out)))
+        return out
+
     def describe(self, chain0: int = 0, n: int | None = None):
         n = self.num_chains() - chain0 if n is None else n
-        out = (ea_chain_desc * n)()
-        check(lib().ea_describe(self._h, chain0, n, out))
-        return [{f: getattr(d, f) for f, _ in ea_chain_desc._fields_} for d in out]
+        names = DESC_DTYPE.names
+        return [dict(zip(names, d)) for d in self._describe(chain0, n).tolist()]
 
     # a5
     def set_ensemble(self, chain0: int, n: int, kind: int, alpha: float = -3.6,
@@ -267,7 +284,7 @@ class Context:
         check(lib().muca_build_ensemble(self._h, chain0, n, kind, alpha, pole, beta))
 
     def _rows(self, chain0, n):
-        return max(d["b_top"] for d in self.describe(chain0, n)) + 1
+        return int(self._describe(chain0, n)["b_top"].max()) + 1
 
     def set_weights(self, chain0: int, lnW: np.ndarray):
         lnW = np.ascontiguousarray(np.atleast_2d(lnW), dtype=np.float64)
@@ -325,8 +342,8 @@ class Context:
         return out
 
     def roundtrips(self, chain0: int = 0, n: int | None = None, reset: bool = False):
-        return [{f: r[f].item() for f in RT_DTYPE.names if f != "pad"}
-                for r in self.roundtrips_array(chain0, n, reset)]
+        names = RT_DTYPE.names  # "pad", the last one, is left out
+        return [dict(zip(names[:-1], r)) for r in self.roundtrips_array(chain0, n, reset).tolist()]
 
     def roundtrips_array(self, chain0: int = 0, n: int | None = None, reset: bool = False, out=None):
         """Round-trip records as a numpy structured array (fields of ea_rt_stats)."""
@@ -337,8 +354,8 @@ class Context:
 
     def state(self, chain0: int = 0, n: int | None = None, spins: bool = True):
         n = self.num_chains() - chain0 if n is None else n
-        descs = self.describe(chain0, n)
-        V = max(d["L"] ** d["dim"] for d in descs)
+        descs = self._describe(chain0, n)
+        V = int((descs["L"].astype(np.int64) ** descs["dim"]).max())
         S = np.zeros((n, V), dtype=np.int8) if spins else None
         E = np.zeros(n, dtype=np.int32)
         t = np.zeros(n, dtype=np.uint64)
@@ -437,10 +454,11 @@ class Context:
 
     def pt_roundtrips(self, reset: bool = False):
         dim, L, n, M = self._pt
-        out = (ea_pt_stats * (n * M))()
-        check(lib().pt_get_roundtrips(self._h, out, int(reset)))
-        return [[{f: getattr(out[r * M + l], f) for f, _ in ea_pt_stats._fields_ if f != "pad"}
-                 for l in range(M)] for r in range(n)]
+        out = np.zeros(n * M, dtype=PT_DTYPE)
+        check(lib().pt_get_roundtrips(self._h, _p(out), int(reset)))
+        names = PT_DTYPE.names[:-1]  # without "pad"
+        rows = [dict(zip(names, x)) for x in out.tolist()]
+        return [rows[r * M:(r + 1) * M] for r in range(n)]
 
     def pt_swap_counts(self):
         M = self._pt[3]
