@@ -391,7 +391,7 @@ __device__ __forceinline__ void walk_chain(const TileDesc &td, int tile, int ch,
                 };
                 rebuild();
                 while (s < N) {
-                    const int base = p - 4;
+                    int base = p - 4;
                     int pos = base + ((lane - base) & 7), lo = 64, hi = -64;
                     uint32_t H = 0u, en = 0u;
                     auto walk = [&]() {
@@ -406,6 +406,12 @@ __device__ __forceinline__ void walk_chain(const TileDesc &td, int tile, int ch,
                             hi = __vimax3_s32(hi, pa, pos);
                         }
                     };
+                    // a segment's end as a byte: its three low bits, its two high bits from bit 4, bit 6 not
+                    // a candidate of the next segment, bit 7 outside the window
+                    auto leave = [&]() {
+                        ends[32 * k + lane] = (unsigned char)(pos + (pos & 0x18) + ((uint32_t)(pos - base) > 7u ? 0x40 : 0) |
+                                                              ((uint32_t)pos >= (uint32_t)kWin ? 0xC0 : 0));
+                    };
                     if (G::NR * HALF > 160 || s + 32 < N) {  // (small passes: not after the last batch)
                         const uint2 next = att[s + 32 + lane];
                         en = next.y;
@@ -416,9 +422,7 @@ __device__ __forceinline__ void walk_chain(const TileDesc &td, int tile, int ch,
                     } else {
                         walk();
                     }
-                    // the end as a byte: its three low bits, its two high bits from bit 4, bit 6 not a
-                    // candidate of the next segment, bit 7 outside the window
-                    ends[32 * k + lane] = (unsigned char)(pos + (pos & 0x18) + ((uint32_t)(pos - base) > 7u ? 0x40 : 0) | ((uint32_t)pos >= (uint32_t)kWin ? 0xC0 : 0));
+                    leave();
                     __syncwarp();
                     const uint4 ma = reinterpret_cast<const uint4 *>(ends + 32 * k)[0], mb = reinterpret_cast<const uint4 *>(ends + 32 * k)[1];
                     const uint32_t v0 = wk_pick(ma.x, ma.y, (uint32_t)(p & 7)), v1 = wk_pick(ma.z, ma.w, v0);
@@ -429,7 +433,6 @@ __device__ __forceinline__ void walk_chain(const TileDesc &td, int tile, int ch,
                     const int los = __shfl_sync(kFull, lo, src), his = __shfl_sync(kFull, hi, src);
                     post();
                     pe = e;
-                    e = en;
                     pH = Hs;
                     plo = los;
                     phi = his;
@@ -437,8 +440,8 @@ __device__ __forceinline__ void walk_chain(const TileDesc &td, int tile, int ch,
                     pst = base + (int)((cs - (uint32_t)base) & 7u);
                     uint32_t ve = v3;
                     int kc = 32;
-                    const bool all = (((v0 | v1 | v2) & 0xC0u) | (v3 & 0x80u)) == 0u;
-                    if (!all) {  // a segment began outside the candidates or left the window
+                    if ((((v0 | v1 | v2) & 0xC0u) | (v3 & 0x80u)) != 0u) {
+                        // a segment began outside the candidates or left the window: the ones before it count
                         ve = v0;
                         kc = (v0 & 0x80u) ? 0 : 8;
                         if ((v0 & 0xC0u) == 0u && !(v1 & 0x80u)) {
@@ -454,7 +457,51 @@ __device__ __forceinline__ void walk_chain(const TileDesc &td, int tile, int ch,
                             plo = 1000000;
                             phi = -1000000;
                         }
+                        // the rest of the batch again, from candidates around the end of the last one that
+                        // counts: its masks stand as long as the window does, and so do the next batch's
+                        while (kc > 0 && kc < 32) {
+                            const int from = (int)((ve & 7u) | ((ve >> 1) & 0x18u)), first = kc >> 3;
+                            if ((uint32_t)(from - kEdge) > (uint32_t)(kWin - 1 - 2 * kEdge)) break;
+                            post();
+                            base = from - 4;
+                            pos = base + ((lane - base) & 7);
+                            lo = 64;
+                            hi = -64;
+                            H = 0u;
+                            walk();
+                            leave();
+                            __syncwarp();
+                            const uint4 ra = reinterpret_cast<const uint4 *>(ends + 32 * k)[0], rb = reinterpret_cast<const uint4 *>(ends + 32 * k)[1];
+                            const uint32_t f = (uint32_t)(from & 7);
+                            const uint32_t u1 = wk_pick(ra.z, ra.w, f);  // segment 1 is the first that can be left
+                            const uint32_t u2 = wk_pick(rb.x, rb.y, first > 1 ? f : u1);
+                            const uint32_t u3 = wk_pick(rb.z, rb.w, first > 2 ? f : u2);
+                            int now = kc;
+                            bool on = true;
+                            if (first <= 1) {
+                                if (!(u1 & 0x80u)) { now = 16; ve = u1; }
+                                on = (u1 & 0xC0u) == 0u;
+                            }
+                            if (first <= 2 && on) {
+                                if (!(u2 & 0x80u)) { now = 24; ve = u2; }
+                                on = (u2 & 0xC0u) == 0u;
+                            }
+                            if (on && !(u3 & 0x80u)) { now = 32; ve = u3; }
+                            const uint32_t cr = seg == first ? f : (seg == 2 ? u1 : u2);
+                            const int src = (lane & 24) | (int)(cr & 7u);
+                            const uint32_t Hr = __shfl_sync(kFull, H, src);
+                            const int lor = __shfl_sync(kFull, lo, src), hir = __shfl_sync(kFull, hi, src);
+                            if (seg >= first && lane < now) {
+                                pH = Hr;
+                                plo = lor;
+                                phi = hir;
+                            }
+                            pst = base + (int)((cr - (uint32_t)base) & 7u);
+                            if (now == kc) break;  // the next segment leaves the window
+                            kc = now;
+                        }
                     }
+                    e = en;
                     int pend = (int)((ve & 7u) | ((ve >> 1) & 0x18u));
                     if (kc == 0) {  // attempt by attempt while the next one cannot leave the window
                         pend = p;
@@ -477,7 +524,7 @@ __device__ __forceinline__ void walk_chain(const TileDesc &td, int tile, int ch,
                     s += kc;
                     p = pend;
                     k ^= 1;
-                    if ((!all || (uint32_t)(pend - kEdge) > (uint32_t)(kWin - 1 - 2 * kEdge)) && s < N) {
+                    if ((kc < 32 || (uint32_t)(pend - kEdge) > (uint32_t)(kWin - 1 - 2 * kEdge)) && s < N) {
                         b = w0 + p;
                         post();
                         rebuild();
