@@ -682,6 +682,31 @@ static ColourPlan colour_plan(const ea_ctx *ctx) {
     return have && t_checker < t_walk ? checker : walk;
 }
 
+// The lexicographic order of full tiles at L >= 7 in parts, a block each (muca_sweep.cu): a full tile
+// reads its thresholds through L1 (100 to 113 cycles per attempt of a chain), a part of 16, 8 or 4 chains
+// has them in shared memory (60 to 75).  Taken while every part has an SM to itself, for tiles of one size
+// class and one block per tile; beyond that the full tiles hold more chains.  Attempts/ns, full tiles ->
+// parts: L = 8, 512 chains 9.7 -> 15.6, 2048 38.1 -> 61.6 (4096, two waves of parts: 74.4 -> 61.8); L = 7,
+// 1024 19.0 -> 28.7; L = 9, 1024 21.2 -> 28.4; L = 10, 1024 21.0 -> 31.4; L = 11, 512 10.3 -> 17.0; L =
+// 12, 512 10.0 -> 18.4 (1024: 19.7 -> 18.4).  At L <= 6 full tiles have their thresholds in shared memory
+// (parts of 16: within 5 %, either way).
+struct PartsPlan {
+    int cls = -1, n_parts = 0;
+    size_t smem = 0;
+};
+
+static PartsPlan parts_plan(const ea_ctx *ctx) {
+    PartsPlan p, none;
+    if (ctx->persistent || ctx->dim != 3 || ctx->tiles.empty()) return none;
+    p.cls = sweep_part_class(ctx->tiles[0].L);
+    for (const TileDesc &td : ctx->tiles) {
+        if (td.width != kTile || p.cls < 0 || sweep_part_class(td.L) != p.cls) return none;
+        p.n_parts = kTile / sweep_part_chains(td.L);
+        p.smem = std::max(p.smem, sweep_part_smem_bytes(td.L));
+    }
+    return (int)ctx->tiles.size() * p.n_parts <= ctx->n_sm ? p : none;
+}
+
 // the context's sweeps in its order and launch configuration, queued on its stream (also the
 // serving loop's tick in the colour order)
 int ctx_enqueue_sweeps(ea_ctx *ctx, uint64_t n_sweeps, int count_roundtrips) {
@@ -707,8 +732,15 @@ int ctx_enqueue_sweeps(ea_ctx *ctx, uint64_t n_sweeps, int count_roundtrips) {
     for (const TileDesc &td : ctx->tiles)
         if (!sweep_width_supported(td.dim, td.L, td.width))
             return fail(EA_EINVAL, "tiles of %d chains at L=%d run only in the colour order", td.width, td.L);
+    const PartsPlan parts = parts_plan(ctx);
     for (uint64_t done = 0; done < n_sweeps; done += chunk) {
         const uint64_t now = std::min(chunk, n_sweeps - done);
+        if (parts.cls >= 0) {
+            EA_CUDA(launch_sweeps_parts(ctx->d_tiles, nt, parts.cls, parts.n_parts, parts.smem, ctx->d_slots,
+                                        ctx->d_spins, ctx->d_bonds, ctx->d_thr, ctx->d_hist, now, ctx->key,
+                                        count_roundtrips, reinterpret_cast<unsigned *>(ctx->d_queue + 1), ctx->stream));
+            continue;
+        }
         if (ctx->persistent) {
             int per_sm = sweep_blocks_per_sm(ctx->dim, ctx->sweep_smem);
             if (ctx->blocks_per_sm > 0) per_sm = std::min(per_sm, ctx->blocks_per_sm);
@@ -810,6 +842,8 @@ extern "C" int ea_graph_capture(ea_ctx *ctx, int n_iter, uint64_t sweeps_per_ite
     EA_CUDA(cudaStreamSynchronize(ctx->stream));
     // attributes are set outside the capture (they are not stream work)
     EA_CUDA(prepare_sweeps(ctx->dim, ctx->sweep_smem));
+    const PartsPlan parts = parts_plan(ctx);
+    if (parts.cls >= 0) EA_CUDA(prepare_parts(parts.cls, parts.smem));
     EA_CUDA(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
     int rc = EA_OK;
     const int nt = (int)ctx->tiles.size();

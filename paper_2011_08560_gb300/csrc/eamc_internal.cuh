@@ -106,6 +106,16 @@ cudaError_t launch_sweeps(const TileDesc *d_tiles, const int32_t *d_tile_list, i
                           const uint32_t *d_bonds, const uint32_t *d_thr, uint32_t *d_hist, uint64_t n_sweeps,
                           PhiloxKey key, int count_rt, unsigned *d_diag, cudaStream_t st);
 int sweep_blocks_per_sm(int dim, size_t smem);
+// the lexicographic sweep of 3D tiles of 32 chains in parts, a block each: the size's kernel class (-1:
+// none), chains and shared memory of a part
+int sweep_part_class(int L);
+int sweep_part_chains(int L);
+size_t sweep_part_smem_bytes(int L);
+cudaError_t prepare_parts(int cls, size_t smem);
+cudaError_t launch_sweeps_parts(const TileDesc *d_tiles, int n_tiles, int cls, int n_parts, size_t smem,
+                                SlotState *d_slots, uint32_t *d_spins, const uint32_t *d_bonds, const uint32_t *d_thr,
+                                uint32_t *d_hist, uint64_t n_sweeps, PhiloxKey key, int count_rt, unsigned *d_diag,
+                                cudaStream_t st);
 // the colour-order sweep, one warp per chain (muca_walk.cu): every L and tile width; d_list: the tiles,
 // longest first
 bool colour_width_supported(int dim, int L, int width);

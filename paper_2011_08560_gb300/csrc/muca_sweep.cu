@@ -82,7 +82,7 @@ __device__ __forceinline__ T rot_prev(T r) {
 
 template <int DIM, int L, int W>
 struct Geo {
-    static_assert(W == 32 || W == 16 || W == 8, "tile width");
+    static_assert(W == 32 || W == 16 || W == 8 || W == 4, "tile width");
     using T = RowT<L>;
     static constexpr int NR = DIM == 3 ? L * L : L;          // rows along x
     static constexpr int V = NR * L;
@@ -145,8 +145,10 @@ __device__ __forceinline__ void get4(const uint4 *slots, int q, int ln, T &a, T 
 // Running LAG rows ahead is exact as long as every row a record reads as final has been swept:
 // besides the -y row (which the consumer adds itself), the last row of a plane (y = L-1) reads
 // the plane's first row, L-1 rows back, so LAG <= L-2; the -z row is L rows back.
-template <int DIM, int L, int W>
-__device__ __forceinline__ void sweep_tile(const TileDesc &td, int tile, SlotState *__restrict__ slots,
+//
+// PART: the block runs W chains of a wider tile, from chain ch0 on (else the whole tile, ch0 = 0).
+template <int DIM, int L, int W, bool PART = false>
+__device__ __forceinline__ void sweep_tile(const TileDesc &td, int tile, int part0, SlotState *__restrict__ slots,
                                            uint32_t *__restrict__ spins,
                                            const uint32_t *__restrict__ bonds,
                                            const uint32_t *__restrict__ thr,
@@ -163,6 +165,7 @@ __device__ __forceinline__ void sweep_tile(const TileDesc &td, int tile, SlotSta
     // first (lane < W, `owner`) writes to global memory
     const int ln = lane & (W - 1);
     const bool owner = lane < W;
+    const int ch0 = PART ? part0 : 0, cl = ch0 + ln;  // cl: the chain's lane in the tile
 
     // ---- stage the lattice as nibble-packed row words, chain-interleaved: word k of chain ln
     //      at [k*W + ln].  Nibble x of a row word is site x of that row.
@@ -180,10 +183,10 @@ __device__ __forceinline__ void sweep_tile(const TileDesc &td, int tile, SlotSta
 #pragma unroll
         for (int x = 0; x < L; ++x) {
             const int i = row * L + x;
-            r |= T((gsp[i] >> ln) & 1u) << (4 * x);
-            jx |= T((gbd[i * DIM + 0] >> ln) & 1u) << (4 * x);
-            jy |= T((gbd[i * DIM + 1] >> ln) & 1u) << (4 * x);
-            if constexpr (DIM == 3) jz |= T((gbd[i * DIM + 2] >> ln) & 1u) << (4 * x);
+            r |= T((gsp[i] >> cl) & 1u) << (4 * x);
+            jx |= T((gbd[i * DIM + 0] >> cl) & 1u) << (4 * x);
+            jy |= T((gbd[i * DIM + 1] >> cl) & 1u) << (4 * x);
+            if constexpr (DIM == 3) jz |= T((gbd[i * DIM + 2] >> cl) & 1u) << (4 * x);
         }
         Rs[row * W + ln] = r;
         JXs[row * W + ln] = jx;
@@ -191,10 +194,10 @@ __device__ __forceinline__ void sweep_tile(const TileDesc &td, int tile, SlotSta
         if constexpr (DIM == 3) JZs[row * W + ln] = jz;
     }
 
-    const int slot = tile * kTile + ln;
+    const int slot = tile * kTile + cl;
     SlotState ss = slots[slot];
     const bool active = ss.active != 0;
-    const uint64_t lrow = td.w_base + (uint64_t)ln * G::B;
+    const uint64_t lrow = td.w_base + (uint64_t)cl * G::B;
     // element (b, n) of this chain's table at byte offset b * RSB + n * NSB from `tab`; rows
     // -DIM .. B-1+DIM are addressable (padding), so a speculative row one move away from a
     // valid row never needs a clamp
@@ -476,10 +479,20 @@ __device__ __forceinline__ void sweep_tile(const TileDesc &td, int tile, SlotSta
     constexpr uint32_t kOwned = W == 32 ? kFull : ((1u << W) - 1u);
     for (int r2 = 0; r2 < NR; ++r2) {
         const T Rw = Rs[r2 * W + ln];
+        uint32_t mine = 0u;  // PART: the word of site `lane`
 #pragma unroll
         for (int x = 0; x < L; ++x) {
             const uint32_t m = __ballot_sync(kFull, ((Rw >> (4 * x)) & 1u) != 0) & kOwned;
-            if (lane == 0) spins[td.spin_off + r2 * L + x] = m;
+            if constexpr (PART) mine = lane == x ? m : mine;
+            else if (lane == 0) spins[td.spin_off + r2 * L + x] = m;
+        }
+        if constexpr (PART) {  // only this block's bits of the word: other blocks write the others
+            if (lane < L) {
+                uint32_t *word = spins + td.spin_off + r2 * L + lane;
+                if constexpr (W == 16) reinterpret_cast<uint16_t *>(word)[ch0 / 16] = (uint16_t)mine;
+                else if constexpr (W == 8) reinterpret_cast<uint8_t *>(word)[ch0 / 8] = (uint8_t)mine;
+                else atomicXor(word, (*word ^ (mine << ch0)) & (kOwned << ch0));
+            }
         }
     }
 }
@@ -503,7 +516,7 @@ __device__ __forceinline__ void sweep_one(const TileDesc *__restrict__ tiles, in
     const TileDesc td = tiles[tile];
     const uint64_t n_tile = n_sweeps * (uint64_t)(td.sweep_mul > 0 ? td.sweep_mul : 1);
 #define EAMC_BODY(LL, WW) \
-    sweep_tile<DIM, LL, WW>(td, tile, slots, spins, bonds, thr, hist, n_tile, key, count_rt, diag, smem_raw)
+    sweep_tile<DIM, LL, WW>(td, tile, 0, slots, spins, bonds, thr, hist, n_tile, key, count_rt, diag, smem_raw)
 #define EAMC_CASE(LL)                                                              \
     case LL:                                                                       \
         if constexpr (width_compiled(DIM, LL, 16)) {                               \
@@ -547,6 +560,38 @@ muca_sweep_kernel(const TileDesc *__restrict__ tiles, const int32_t *__restrict_
                        smem_raw);
         __syncthreads();  // every warp is done with this tile's shared memory
     }
+}
+
+// A tile of 32 chains in parts, a block each, so that a part's thresholds fit in shared memory: 16 chains
+// for L = 7, 8, 8 for L = 9, 10, 4 for L = 11, 12 (3D).  One kernel per class of sizes (0: L = 7, 8, 1: 9,
+// 10, 2: 11, 12) with registers of its own (96, 106, 121; the kernel of every size needs 254).
+__host__ __device__ constexpr int part_class(int L) { return L <= 6 ? -1 : L <= 8 ? 0 : L <= 10 ? 1 : 2; }
+
+template <int CLASS>
+__global__ void __launch_bounds__(kThreads, 1)
+muca_parts_kernel(const TileDesc *__restrict__ tiles, int n_parts, SlotState *__restrict__ slots,
+                  uint32_t *__restrict__ spins, const uint32_t *__restrict__ bonds, const uint32_t *__restrict__ thr,
+                  uint32_t *__restrict__ hist, uint64_t n_sweeps, PhiloxKey key, int count_rt,
+                  unsigned *__restrict__ diag) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int W = CLASS == 0 ? 16 : CLASS == 1 ? 8 : 4;
+    const int tile = blockIdx.x / n_parts, ch0 = blockIdx.x % n_parts * W;
+    const TileDesc td = tiles[tile];
+    if (ch0 >= td.width) return;
+    const uint64_t n_tile = n_sweeps * (uint64_t)(td.sweep_mul > 0 ? td.sweep_mul : 1);
+#define EAMC_PART(LL) \
+    if (td.L == LL) sweep_tile<3, LL, W, true>(td, tile, ch0, slots, spins, bonds, thr, hist, n_tile, key, count_rt, diag, smem_raw)
+    if constexpr (CLASS == 0) {
+        EAMC_PART(7);
+        EAMC_PART(8);
+    } else if constexpr (CLASS == 1) {
+        EAMC_PART(9);
+        EAMC_PART(10);
+    } else {
+        EAMC_PART(11);
+        EAMC_PART(12);
+    }
+#undef EAMC_PART
 }
 
 template <int DIM, int W>
@@ -631,6 +676,48 @@ cudaError_t launch_sweeps(const TileDesc *d_tiles, const int32_t *d_tile_list, i
         muca_sweep_kernel<2><<<n_blocks, kThreads, smem, st>>>(d_tiles, d_tile_list, n_work, d_queue, d_slots, d_spins,
                                                          d_bonds, d_thr, d_hist, n_sweeps, key, count_rt, d_diag);
     }
+    return cudaGetLastError();
+}
+
+int sweep_part_class(int L) { return part_class(L); }
+
+int sweep_part_chains(int L) { return L <= 8 ? 16 : L <= 10 ? 8 : 4; }
+
+size_t sweep_part_smem_bytes(int L) {
+    return L <= 8 ? smem_for_w<3, 16>(L) : L <= 10 ? smem_for_w<3, 8>(L) : smem_for_w<3, 4>(L);
+}
+
+static const void *parts_kernel(int cls) {
+    const void *k[3] = {(const void *)muca_parts_kernel<0>, (const void *)muca_parts_kernel<1>,
+                        (const void *)muca_parts_kernel<2>};
+    return k[cls];
+}
+
+cudaError_t prepare_parts(int cls, size_t smem) {
+    static size_t set_limit[3] = {0, 0, 0};
+    if (smem <= set_limit[cls]) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(parts_kernel(cls), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) set_limit[cls] = smem;
+    return e;
+}
+
+cudaError_t launch_sweeps_parts(const TileDesc *d_tiles, int n_tiles, int cls, int n_parts, size_t smem,
+                                SlotState *d_slots, uint32_t *d_spins, const uint32_t *d_bonds, const uint32_t *d_thr,
+                                uint32_t *d_hist, uint64_t n_sweeps, PhiloxKey key, int count_rt, unsigned *d_diag,
+                                cudaStream_t st) {
+    if (n_tiles <= 0 || n_sweeps == 0) return cudaSuccess;
+    const cudaError_t e = prepare_parts(cls, smem);
+    if (e != cudaSuccess) return e;
+    const int grid = n_tiles * n_parts;
+#define EAMC_PARTS(C) \
+    case C: muca_parts_kernel<C><<<grid, kThreads, smem, st>>>(d_tiles, n_parts, d_slots, d_spins, d_bonds, d_thr, d_hist, n_sweeps, key, count_rt, d_diag); break
+    switch (cls) {
+        EAMC_PARTS(0);
+        EAMC_PARTS(1);
+        EAMC_PARTS(2);
+        default: return cudaErrorInvalidValue;
+    }
+#undef EAMC_PARTS
     return cudaGetLastError();
 }
 

@@ -1,0 +1,32 @@
+"""Full tiles swept in parts, a block each (lexicographic order, L >= 7), against the same tiles whole
+(whose trajectories the other tests hold against the oracle)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("L,n", [(7, 33), (8, 70), (8, 2432), (9, 40), (10, 65), (11, 35), (12, 37)])
+def test_full_tiles_in_parts_agree(L, n):
+    """Lexicographic order: full tiles run in parts of 16, 8 or 4 chains while each part has an SM to
+    itself; the work-queue launch runs them whole.  Same chains, same results, last tiles ragged."""
+    from paper_2011_08560_gb300 import eamc
+
+    def run(persistent):
+        ctx = eamc.Context(seed=31)
+        ctx.init_disorder(3, L, n, rid0=7)
+        ctx.set_ensemble(0, n, eamc.EA_POWERLAW)
+        ctx.set_launch(persistent=persistent)
+        for _ in range(2):
+            ctx.run_sweeps(5)
+            ctx.update_weights()
+        ctx.run_sweeps(4, count_roundtrips=True)
+        ctx.check()
+        return ctx
+
+    parts, whole = run(False), run(True)
+    for a, b in zip(parts.state(), whole.state()):
+        assert np.array_equal(a, b)
+    assert np.array_equal(parts.histograms(), whole.histograms())
+    assert np.array_equal(parts.roundtrips_array(), whole.roundtrips_array())
+    assert np.array_equal(parts.get_weights(), whole.get_weights())
