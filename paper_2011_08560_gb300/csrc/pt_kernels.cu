@@ -218,8 +218,7 @@ __global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
     // round-trip records of the replicas in the CTA's slots, for the launch; an exchange moves them with
     // the configurations
     PtRt *Rh = reinterpret_cast<PtRt *>(Db + spc * 32);    // [spc][32]
-    float *Df = reinterpret_cast<float *>(Rh + spc * 32);  // [spc][32] Db in single precision
-    int32_t *Cl = (int32_t *)(Df + spc * 32);  // odd L: sites by colour [V], then offsets [4]
+    int32_t *Cl = (int32_t *)(Rh + spc * 32);  // odd L: sites by colour [V], then offsets [4]
 
     const uint32_t group_rid0 = a.rid0 + 32u * (uint32_t)g;
     const int nvalid = min(32, a.n_real - 32 * g);
@@ -240,7 +239,6 @@ __global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
     for (int q = tid; q < spc * 32; q += blockDim.x) {
         const int k = k0 + (q >> 5), b = q & 31;
         Db[q] = (k + 1 < M) ? a.beta[((size_t)g * M + k + 1) * 32 + b] - a.beta[((size_t)g * M + k) * 32 + b] : 0.0;
-        Df[q] = (float)Db[q];
         Xc[q] = 0u;
     }
     for (int q = tid; q < 64; q += blockDim.x) Bd[q] = a.bounds[(size_t)g * 64 + q];
@@ -460,7 +458,7 @@ __global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
                 // p = exp(-x), quantised to 32 bits.  In single precision p is known to 1e-5; the exact
                 // threshold (FP64, 32 times slower) is needed only where the word lies that close to it
                 const int d4 = (e0 - e1) / 4;
-                const float x = Df[ks * 32 + lane] * (4.0f * (float)d4), pf = expf(-x) * 4294967296.0f, wf = (float)w.x;
+                const float x = (float)Db[ks * 32 + lane] * (4.0f * (float)d4), pf = expf(-x) * 4294967296.0f, wf = (float)w.x;
                 const float slack = (2e-6f + 1e-6f * x) * pf + 1e-6f * wf + 4.0f;
                 ok = wf < pf;
                 if (!(fabsf(wf - pf) > slack)) {
@@ -665,7 +663,7 @@ cudaError_t pt_launch_all(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, u
     const int threads = G::threads(a.spc);
     const size_t smem = (size_t)(a.spc * 128 + a.spc * G::V + G::NB + a.spc * 32 * 2 + a.spc +
                                  (threads / 32) * (kTailQ * 6 + a.spc * 32) + a.spc * 32 + 64 + 1 + 2 * a.spc * 32 +
-                                 a.spc * 32 * (int)(sizeof(PtRt) / 4) + a.spc * 32 + ((L & 1) ? G::V + 4 : 0)) * 4;
+                                 a.spc * 32 * (int)(sizeof(PtRt) / 4) + ((L & 1) ? G::V + 4 : 0)) * 4;
     cudaError_t e = cudaFuncSetAttribute(pt_kernel<DIM, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(pt_kernel<DIM, L>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
