@@ -198,6 +198,8 @@ __global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
     const int rank = (int)cluster.block_rank();
     const int g = blockIdx.x / (int)cluster.num_blocks();
     const int spc = a.spc, k0 = rank * spc, M = a.M;
+    // slots of this CTA: the last one may have fewer than spc, and sweeps empty ones (zeroed) for the rest
+    const int mine = min(spc, M - k0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
 
     constexpr int NCOL = (L & 1) ? 3 : 2;
@@ -225,18 +227,19 @@ __global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
     const uint32_t valid = nvalid >= 32 ? kFull : ((1u << nvalid) - 1u);
 
     for (int k = tid; k < spc * V; k += blockDim.x)
-        S[k] = a.spins[((size_t)g * M + k0) * V + k];
+        S[k] = k < mine * V ? a.spins[((size_t)g * M + k0) * V + k] : 0u;
     for (int k = tid; k < NB; k += blockDim.x) J[k] = a.bonds[(size_t)g * NB + k];
-    for (int k = tid; k < spc * 32; k += blockDim.x) {
+    for (int k = tid; k < mine * 32; k += blockDim.x) {
         Es[k] = a.E[((size_t)g * M + k0) * 32 + k];
         const int label = a.label[((size_t)g * M + k0) * 32 + k];
         Ls[k] = label;
         Rh[k] = a.rt[((size_t)g * M + label) * 32 + (k & 31)];
     }
-    for (int k = tid; k < spc * 128; k += blockDim.x) sm[k] = a.planes[((size_t)g * M + k0) * 128 + k];
+    for (int k = tid; k < spc * 128; k += blockDim.x)
+        sm[k] = k < mine * 128 ? a.planes[((size_t)g * M + k0) * 128 + k] : 0u;
     // per launch: beta_{k+1} - beta_k of every owned pair and realization, the round-trip bounds,
     // zeroed exchange counters (added to the global ones at the end)
-    for (int q = tid; q < spc * 32; q += blockDim.x) {
+    for (int q = tid; q < mine * 32; q += blockDim.x) {
         const int k = k0 + (q >> 5), b = q & 31;
         Db[q] = (k + 1 < M) ? a.beta[((size_t)g * M + k + 1) * 32 + b] - a.beta[((size_t)g * M + k) * 32 + b] : 0.0;
         Xc[q] = 0u;
@@ -434,7 +437,7 @@ __global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
             __syncthreads();
         }
         // ---- energies of the owned slots from the warps' sums
-        for (int k = tid; k < spc * 32; k += blockDim.x) {
+        for (int k = tid; k < mine * 32; k += blockDim.x) {
             int u = 0;
 #pragma unroll
             for (int w = 0; w < G::JT / 32; ++w) u += Ep[w * spc * 32 + k];
@@ -534,7 +537,7 @@ __global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
         }
         cluster.sync();  // exchanges complete everywhere
         // ---- round trips / lowest energy per replica; its record travels with it
-        for (int q = tid; q < spc * 32; q += blockDim.x) {
+        for (int q = tid; q < mine * 32; q += blockDim.x) {
             const int b = q & 31;
             if (!((valid >> b) & 1u)) continue;
             const int E = Es[q];
@@ -556,16 +559,16 @@ __global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
     }
     __syncthreads();
     // ---- write back; a replica's record to its label
-    for (int q = tid; q < spc * 32; q += blockDim.x) a.rt[((size_t)g * M + Ls[q]) * 32 + (q & 31)] = Rh[q];
-    for (int q = tid; q < spc * 32; q += blockDim.x) {
+    for (int q = tid; q < mine * 32; q += blockDim.x) a.rt[((size_t)g * M + Ls[q]) * 32 + (q & 31)] = Rh[q];
+    for (int q = tid; q < mine * 32; q += blockDim.x) {
         const int k = k0 + (q >> 5);
         if (Xc[q]) {
             a.xacc[((size_t)g * M + k) * 32 + (q & 31)] += Xc[q];
             atomicAdd(&a.swaps[k], (unsigned long long)Xc[q]);
         }
     }
-    for (int k = tid; k < spc * V; k += blockDim.x) a.spins[((size_t)g * M + k0) * V + k] = S[k];
-    for (int k = tid; k < spc * 32; k += blockDim.x) {
+    for (int k = tid; k < mine * V; k += blockDim.x) a.spins[((size_t)g * M + k0) * V + k] = S[k];
+    for (int k = tid; k < mine * 32; k += blockDim.x) {
         a.E[((size_t)g * M + k0) * 32 + k] = Es[k];
         a.label[((size_t)g * M + k0) * 32 + k] = Ls[k];
     }
@@ -653,7 +656,7 @@ cudaError_t pt_launch_all(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, u
     a.xacc = p->d_xacc;
     a.swaps = p->d_swaps;
     a.M = p->M;
-    a.spc = p->M / p->cs;
+    a.spc = (p->M + p->cs - 1) / p->cs;
     a.n_real = p->n_real;
     a.rid0 = p->rid0;
     a.t0 = p->t;
@@ -693,6 +696,36 @@ cudaError_t pt_dispatch(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, uin
     PT_CASE(2, 10) PT_CASE(2, 11) PT_CASE(2, 12)
 #undef PT_CASE
     return cudaErrorInvalidValue;
+}
+
+// passes over its slots that a CTA of spc slots makes in a colour
+int pt_passes(int dim, int L, int spc) {
+#define PT_CASE(D, LL) \
+    if (dim == D && L == LL) return (spc + PtGeo<D, LL>::kt(spc) - 1) / PtGeo<D, LL>::kt(spc);
+    PT_CASE(3, 3) PT_CASE(3, 4) PT_CASE(3, 5) PT_CASE(3, 6) PT_CASE(3, 7) PT_CASE(3, 8) PT_CASE(3, 9)
+    PT_CASE(3, 10) PT_CASE(3, 11) PT_CASE(3, 12)
+    PT_CASE(2, 3) PT_CASE(2, 4) PT_CASE(2, 5) PT_CASE(2, 6) PT_CASE(2, 7) PT_CASE(2, 8) PT_CASE(2, 9)
+    PT_CASE(2, 10) PT_CASE(2, 11) PT_CASE(2, 12)
+#undef PT_CASE
+    return spc;
+}
+
+// CTAs per realization group, at most 8 (clusters of 16 measured slower): the largest number that divides
+// the slots, or the one with the fewest slots to a CTA, whose last CTA sweeps some empty ones.  A sweep
+// takes about passes x max(1, CTAs / SMs); the second has to win by a quarter, as empty slots and smaller
+// blocks cost it up to that.  us per sweep, dividing -> fewest: M = 17, L = 7, 256 realizations 23.7 -> 7.9;
+// L = 8, 1024 28.7 -> 8.8; L = 12, 256 104 -> 18; L = 4, 1024 6.0 -> 3.7; M = 20, L = 10, 256 13.7 -> 10.8;
+// M = 13, L = 8, 600 21.0 -> 6.8.  Left dividing: M = 17, L = 4, 8192 9.5 (11.2); M = 20, L = 6, 1024 6.8
+// (7.5), L = 8, 2048 16.6 (17.4).
+int pt_cluster(int dim, int L, int M, int n_groups, int n_sm) {
+    int even = 1;
+    for (int c = 8; c >= 2 && even == 1; --c)
+        if (M % c == 0) even = c;
+    const int spc = (M + 7) / 8, least = (M + spc - 1) / spc;
+    auto cost = [&](int cs) {
+        return (long long)pt_passes(dim, L, (M + cs - 1) / cs) * std::max((long long)n_sm, (long long)n_groups * cs);
+    };
+    return 4 * cost(even) >= 5 * cost(least) ? least : even;
 }
 
 // Metropolis threshold planes of every (group, slot): one warp, lane b = realization bit.
@@ -823,11 +856,7 @@ extern "C" int pt_init(ea_ctx *ctx, int dim, int L, int n_real, uint32_t rid0, i
     p->n_real = n_real;
     p->n_groups = (n_real + 31) / 32;
     p->rid0 = rid0;
-    p->cs = 1;
-    // the largest cluster (at most 8 CTAs: 16-CTA clusters measured slower) that splits the
-    // slots evenly, for the most CTAs per realization group
-    for (int c = 8; c >= 2; --c)
-        if (M % c == 0) { p->cs = c; break; }
+    p->cs = pt_cluster(dim, L, M, p->n_groups, ctx->n_sm);
     const size_t G = p->n_groups;
     auto alloc = [&](void **ptr, size_t bytes) -> int {
         if (cudaMalloc(ptr, bytes) != cudaSuccess) return fail(EA_ENOMEM, "PT allocation of %zu bytes failed", bytes);
