@@ -25,10 +25,10 @@
 // between the colour passes a CTA walks a chain of short steps (open comparisons, energies, exchange)
 // whose latencies add up: 13 of 29 thousand cycles a sweep before they were shortened, 7 now.
 // us per sweep, before -> now: 1024 x 32 of L = 8 15.9 -> 11.6 (1056 -> 1447 attempts/ns); 32 x 32 of
-// L = 8 11.3 -> 7.1; 1024 x 14 of L = 6 7.4 -> 5.3; 128 x 20 of L = 12 35 -> 23; 333 x 12 of L = 5 6.7 ->
-// 4.6; 256 x 17 of L = 7 36 -> 24.
+// L = 8 11.3 -> 6.7; 1024 x 14 of L = 6 7.4 -> 5.3; 128 x 20 of L = 12 35 -> 16; 333 x 12 of L = 5 6.7 ->
+// 4.6; 256 x 17 of L = 7 36 -> 7.9.
 //
-// Parallel work.  One thread-block cluster per group: CS CTAs, each owning M/CS consecutive
+// Parallel work.  One thread-block cluster per group: CS CTAs, each owning M/CS (rounded up) consecutive
 // slots in shared memory; a thread keeps its sites (index, neighbours, bonds) and goes through
 // the slots.  Energies come from the updates themselves (bit-sliced counts, warp bit-matrix
 // transpose, popcount): for even L the unsatisfied bonds counted at the second colour's sites, for
@@ -101,7 +101,10 @@ __device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
     return x;
 }
 
-template <int DIM, int L>
+constexpr int kTailQ = 32;  // open comparisons a warp defers per colour phase
+constexpr size_t kPtSmemMax = 227u << 10;  // shared memory of a block
+
+template <int DIM, int L, bool WIDE = false>
 struct PtGeo {
     static constexpr int NR = DIM == 3 ? L * L : L;
     static constexpr int V = NR * L;
@@ -130,12 +133,19 @@ struct PtGeo {
     }
     static constexpr int NC = ODD ? most_odd() : HALF;
     // a block's threads: JT over the sites of a colour (whole warps, in NP passes where the sites are more
-    // than 288), times KT slots side by side
-    static constexpr int NP = (NC + 287) / 288;
+    // than MAX), times KT slots side by side.  At most 288 threads, two blocks to an SM; the wide form
+    // (WIDE: at most 576, one block to an SM) is for batches whose CTAs have an SM each, which wait for
+    // latencies, not for pipes
+    static constexpr int MAX = WIDE ? 576 : 288;
+    static constexpr int NP = (NC + MAX - 1) / MAX;
     static constexpr int JT = ((NC + NP - 1) / NP + 31) / 32 * 32;
-    static constexpr int KT_MAX = JT > 128 ? 1 : 256 / JT;
+    static constexpr int KT_MAX = WIDE ? MAX / JT : (JT > 128 ? 1 : 256 / JT);
     static __host__ __device__ constexpr int kt(int spc) { return spc < KT_MAX ? spc : KT_MAX; }
     static __host__ __device__ constexpr int threads(int spc) { return JT * kt(spc); }
+    static constexpr size_t smem(int spc) {
+        return (size_t)(spc * 128 + spc * V + NB + spc * 32 * 2 + spc + (threads(spc) / 32) * (kTailQ * 6 + spc * 32) +
+                        spc * 32 + 64 + 1 + 2 * spc * 32 + spc * 32 * (int)(sizeof(PtRt) / 4) + (ODD ? V + 4 : 0)) * 4;
+    }
 };
 
 // neighbour of site i along axis d (0 x, 1 y, 2 z), direction +1 / -1
@@ -169,8 +179,6 @@ __device__ __forceinline__ uint32_t quantize_prob(double p) {
     return (q >= 4294967294.0) ? 0xFFFFFFFEu : (uint32_t)q;
 }
 
-constexpr int kTailQ = 32;  // open comparisons a warp defers per colour phase
-
 struct PtArgs {
     uint32_t *spins;
     const uint32_t *bonds;
@@ -189,9 +197,9 @@ struct PtArgs {
     PhiloxKey key;
 };
 
-template <int DIM, int L>
-__global__ void __launch_bounds__(288, 2) pt_kernel(PtArgs a) {
-    using G = PtGeo<DIM, L>;
+template <int DIM, int L, bool WIDE>
+__global__ void __launch_bounds__(PtGeo<DIM, L, WIDE>::MAX, WIDE ? 1 : 2) pt_kernel(PtArgs a) {
+    using G = PtGeo<DIM, L, WIDE>;
     constexpr int V = G::V, NB = G::NB, HALF = G::HALF;
     constexpr bool ODD = G::ODD;
     cg::cluster_group cluster = cg::this_cluster();
@@ -634,6 +642,31 @@ __global__ void pt_energy_kernel(const uint32_t *spins, const uint32_t *bonds, i
     E[((size_t)g * M + k) * 32 + lane] = 2 * u - NB;
 }
 
+template <int DIM, int L, bool WIDE>
+cudaError_t pt_launch_sweeps(const PtState *p, const PtArgs &a, cudaStream_t st) {
+    using G = PtGeo<DIM, L, WIDE>;
+    const int threads = G::threads(a.spc);
+    const size_t smem = G::smem(a.spc);
+    cudaError_t e = cudaFuncSetAttribute(pt_kernel<DIM, L, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(pt_kernel<DIM, L, WIDE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(p->n_groups * p->cs);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = p->cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, pt_kernel<DIM, L, WIDE>, a);
+}
+
 template <int DIM, int L>
 cudaError_t pt_launch_all(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, uint64_t n_sweeps,
                           int count_rt) {
@@ -663,28 +696,20 @@ cudaError_t pt_launch_all(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, u
     a.n_sweeps = n_sweeps;
     a.count_rt = count_rt;
     a.key = ctx->key;
-    const int threads = G::threads(a.spc);
-    const size_t smem = (size_t)(a.spc * 128 + a.spc * G::V + G::NB + a.spc * 32 * 2 + a.spc +
-                                 (threads / 32) * (kTailQ * 6 + a.spc * 32) + a.spc * 32 + 64 + 1 + 2 * a.spc * 32 +
-                                 a.spc * 32 * (int)(sizeof(PtRt) / 4) + ((L & 1) ? G::V + 4 : 0)) * 4;
-    cudaError_t e = cudaFuncSetAttribute(pt_kernel<DIM, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(pt_kernel<DIM, L>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg;
-    std::memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(p->n_groups * p->cs);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = ctx->stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = p->cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, pt_kernel<DIM, L>, a);
+    // the wide form from 3D L = 8 while the clusters fit the SMs with a CTA to each (a cluster of 8 stays
+    // within a GPC: 15 of them fit, so the line is three quarters of the SMs).  us per sweep, narrow ->
+    // wide: L = 8, 448 x 32 7.16 -> 6.75; L = 9, 64 x 32 12.5 -> 11.6; L = 10, 256 x 14 8.0 -> 6.9; L = 11,
+    // 128 x 20 21.0 -> 17.4; L = 12, 448 x 32 24.3 -> 20.0.  Beyond the line two narrow CTAs share an SM:
+    // L = 8, 512 x 32 10.6 (wide 13.4); L = 9, 608 x 32 19.4 (25.0).  Below L = 8 the sites of a colour fill
+    // 128 threads at most and slots lie side by side already: L = 6, 200 x 32 4.75 (5.17), L = 7, 448 x 20
+    // 8.0 (8.3)
+    if constexpr (DIM == 3 && L >= 8) {
+        using W = PtGeo<DIM, L, true>;
+        if (4 * p->n_groups * p->cs <= 3 * ctx->n_sm && W::threads(a.spc) > G::threads(a.spc) &&
+            W::smem(a.spc) <= kPtSmemMax)
+            return pt_launch_sweeps<DIM, L, true>(p, a, ctx->stream);
+    }
+    return pt_launch_sweeps<DIM, L, false>(p, a, ctx->stream);
 }
 
 cudaError_t pt_dispatch(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, uint64_t n_sweeps, int count_rt) {
