@@ -455,6 +455,8 @@ extern "C" int ea_init_disorder(ea_ctx *ctx, int dim, int L, int n, uint32_t rid
         ctx->chain_woff.push_back(nt[k / W].w_base + (uint64_t)(k % W) * B);
         ctx->chain_btop.push_back(0);
     }
+    ctx->chain_power.resize(ctx->chain_slot.size(), 0);
+    ctx->weight_steps = 0;
     if ((rc = ctx_refresh_chains(ctx))) return rc;
     if ((rc = ctx_rebuild_order(ctx))) return rc;
     // flat weights (ln W = 0 already) -> thresholds
@@ -499,6 +501,7 @@ extern "C" int muca_set_ensemble(ea_ctx *ctx, int chain0, int n, int kind, doubl
                                                                 pole_dE, beta);
     EA_CUDA(cudaGetLastError());
     EA_CUDA(cudaStreamSynchronize(ctx->stream));
+    for (int k = 0; k < n; ++k) ctx->set_power(chain0 + k, kind == EA_POWERLAW);
     return EA_OK;
 }
 
@@ -571,6 +574,7 @@ extern "C" int muca_set_weights(ea_ctx *ctx, int chain0, int n, const double *ln
     int rc = table_io<double>(ctx, chain0, n, ctx ? ctx->d_lnW : nullptr, 1, const_cast<double *>(lnW),
                               stride, true);
     if (rc) return rc;
+    ctx->weights_given();
     EA_CUDA(launch_quantize(ctx->d_tiles, (int)ctx->tiles.size(), ctx->d_slots, ctx->d_lnW, ctx->d_thr,
                             ctx->stream));
     return EA_OK;
@@ -590,6 +594,7 @@ extern "C" int muca_set_thresholds(ea_ctx *ctx, int chain0, int n, const uint32_
                                 stride, true);
     if (rc) return rc;
     ctx->thr_injected = true;
+    ctx->weights_given();
     EA_CUDA(launch_enforce_walls(ctx->d_tiles, (int)ctx->tiles.size(), ctx->d_slots, ctx->d_thr, ctx->stream));
     EA_CUDA(cudaStreamSynchronize(ctx->stream));
     return EA_OK;
@@ -641,13 +646,16 @@ extern "C" int muca_set_eg(ea_ctx *ctx, int chain0, int n, const int32_t *e_g) {
 // slower as chains share schedulers) and one lane per chain (muca_checker.cu: 45 to 220 cycles by
 // size and tile width, the same for every chain of a block, one block per SM).  The plan estimates
 // both times of a launch, in cycles, and takes the shorter:
-//   walk:    f (23 a_max + 10.2 sum of a / schedulers), a = attempts of a chain, f by L; fitted to
-//            512 .. 16384 chains of every L between hot chains (first iterations, one third more) and
-//            cold ones (production, one fifth less);
+//   walk:    f h (23 a_max + 10.2 sum of a / schedulers), a = attempts of a chain, f by L, fitted to
+//            512 .. 16384 chains; h: a walk moves fast while attempts are refused, as in the low energies
+//            that a power-law chain reaches after some weight steps (0.92), and slows where most are
+//            accepted, in first steps and flat ensembles (1.2; at L <= 5 no difference);
 //   checker: cycles(L, width) a per wave of one block per SM, as measured.
-// The line lies near 2000 to 4000 chains in full tiles.  Both sides, attempts/ns (walk hot .. cold /
-// checker): L = 8 in tiles of 16, 1024 chains 53 .. 76 / 45, 2048 69 .. 95 / 89, 4096 80 .. 109 / 89;
-// L = 6 in full tiles, 1024 47 / 33, 2048 63 .. 70 / 65, 4096 73 / 130; L = 4, 2048 57 / 42, 4096 65 / 84.
+// Both sides, attempts/ns, walk / checker.  L = 8 in tiles of 16, 4096 power-law chains after 1, 10, 20,
+// 40 weight steps 68, 81, 90, 100 / 89, flat ones 68 to 76 / 89; 2048 58 to 83 / 88; 1024 53 to 76 / 45.
+// L = 6 in full tiles, 2048 50, 61, 66, 69 / 65, flat 50 to 57 / 65; 4096 59 to 83 / 130; 1024 47 / 33.
+// L = 10, 4096 58 to 80 / 78; 1024 39 to 55 / 21.  L = 12, 4096 61 to 82 / 70 to 80.  L = 7 in tiles of 16,
+// 2048 50 to 74 / 51.  L = 5, 4096 56 / 58; 2048 50 / 29.  L = 4, 4096 65 / 84; 2048 57 / 42.
 struct ColourPlan {
     bool walk = true;
     size_t smem = 0;
@@ -655,15 +663,17 @@ struct ColourPlan {
 };
 
 static ColourPlan colour_plan(const ea_ctx *ctx) {
-    static const double f_walk[13] = {0, 0, 0, 4.1, 1.27, 1.4, 1.09, 1.13, 1.0, 1.15, 1.28, 1.28, 1.18};
+    static const double f_walk[13] = {0, 0, 0, 4.1, 1.4, 1.6, 1.09, 1.13, 1.0, 1.15, 1.28, 1.28, 1.18};
     static const double c_full[13] = {0, 0, 0, 220, 100, 146, 64.5, 155, 101, 125, 104, 137, 111};
     static const double c_half[13] = {0, 0, 0, 0, 79, 113, 60.5, 83, 47.5, 0, 0, 0, 0};
     ColourPlan walk, checker;
     checker.walk = false;
+    const bool low = 2 * (size_t)ctx->n_power >= ctx->chain_slot.size() && ctx->weight_steps >= ea_ctx::kIteratedSteps;
+    const double h = low ? 0.92 : 1.2;
     bool have = true;  // the checker kernel has every tile's width
     double w_max = 0, w_sum = 0, c_max = 0, c_sum = 0;
     for (const TileDesc &td : ctx->tiles) {
-        const double a = (double)td.V * std::max(1, td.sweep_mul), f = td.dim == 3 ? f_walk[td.L] : 1.5;
+        const double a = (double)td.V * std::max(1, td.sweep_mul), f = td.dim == 3 ? f_walk[td.L] * (td.L > 5 ? h : 1.0) : 1.5;
         walk.smem = std::max(walk.smem, walk_smem_bytes(td.dim, td.L));
         walk.max_width = std::max(walk.max_width, (int)td.width);
         w_max = std::max(w_max, f * a);
@@ -894,6 +904,7 @@ extern "C" int muca_update_weights(ea_ctx *ctx) {
     const int nt = (int)ctx->tiles.size();
     EA_CUDA(launch_update_weights(ctx->d_tiles, nt, ctx->d_slots, ctx->d_lnW, ctx->d_hist, ctx->d_acc, ctx->stream));
     EA_CUDA(launch_quantize(ctx->d_tiles, nt, ctx->d_slots, ctx->d_lnW, ctx->d_thr, ctx->stream));
+    ctx->weight_steps = std::min(ctx->weight_steps + 1, ea_ctx::kIteratedSteps);
     return EA_OK;
 }
 
@@ -920,6 +931,8 @@ extern "C" int muca_build_ensemble(ea_ctx *ctx, int chain0, int n, int kind, dou
     const int nt = (int)ctx->tiles.size();
     EA_CUDA(launch_build_ensemble(ctx->d_tiles, nt, ctx->d_slots, d_sel, kind, alpha, pole_dE, beta,
                                   ctx->d_lnW, ctx->stream));
+    for (int k = 0; k < n; ++k) ctx->set_power(chain0 + k, kind == EA_POWERLAW);
+    ctx->weights_given();
     // the other chains' thresholds are those of their weights already, unless injected ones are about
     // (2304 chains of L = 6, 128 of them built: 0.12 -> 0.01 ms a call)
     if (ctx->thr_injected) {
@@ -1043,6 +1056,7 @@ extern "C" int muca_copy_weights(ea_ctx *ctx, const int32_t *src, const int32_t 
     int32_t *d_meta = (int32_t *)((char *)scr + ((off.size() * 8 + 255) & ~(size_t)255));
     EA_CUDA(cudaMemcpyAsync(d_off, off.data(), off.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
     EA_CUDA(cudaMemcpyAsync(d_meta, meta.data(), meta.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
+    ctx->weights_given();
     copy_weights_kernel<<<n, 128, 0, ctx->stream>>>(ctx->d_slots, ctx->d_lnW, d_meta, d_off, n);
     EA_CUDA(cudaGetLastError());
     EA_CUDA(launch_quantize(ctx->d_tiles, (int)ctx->tiles.size(), ctx->d_slots, ctx->d_lnW, ctx->d_thr,
@@ -1225,6 +1239,7 @@ extern "C" int ea_snapshot_load(ea_ctx *ctx, const void *buf, size_t size) {
     std::memcpy(cslot.data(), p, h.n_chains * 4); p += h.n_chains * 4;
     std::memcpy(cwoff.data(), p, h.n_chains * 8); p += h.n_chains * 8;
     std::memcpy(cbtop.data(), p, h.n_chains * 4); p += h.n_chains * 4;
+    const char *slots = p;
     int rc;
     if ((rc = grow(&ctx->d_tiles, &ctx->tiles_cap, 0, h.n_tiles, ctx->stream)) ||
         (rc = grow(&ctx->d_slots, &ctx->slots_cap, 0, h.n_tiles * kTile, ctx->stream)) ||
@@ -1261,5 +1276,14 @@ extern "C" int ea_snapshot_load(ea_ctx *ctx, const void *buf, size_t size) {
     ctx->max_V = h.max_V;
     ctx->sweep_smem = h.sweep_smem;
     ctx->thr_injected = true;  // a snapshot may hold injected thresholds
+    ctx->weights_given();
+    ctx->chain_power.assign(h.n_chains, 0);
+    ctx->n_power = 0;
+    for (size_t c = 0; c < h.n_chains; ++c) {
+        if (cslot[c] < 0 || (size_t)cslot[c] >= h.n_tiles * kTile) continue;
+        SlotState s;
+        std::memcpy(&s, slots + (size_t)cslot[c] * sizeof(SlotState), sizeof s);
+        ctx->set_power((int)c, s.kind == EA_POWERLAW);
+    }
     return ctx_rebuild_order(ctx);
 }

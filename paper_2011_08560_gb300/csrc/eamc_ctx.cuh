@@ -20,6 +20,16 @@ struct ea_ctx {
     uint64_t max_t_host = 0;  // upper bound of every chain's sweep counter
     bool thr_injected = false;  // some chain's thresholds may not be its weights' (muca_set_thresholds,
                                 // a snapshot): the next re-quantisation takes every chain
+    // what the colour order's choice of kernel goes by (speed only): the power-law chains, and the weight
+    // steps since the newest chains were made, given weights counted as kIteratedSteps of them
+    std::vector<uint8_t> chain_power;
+    int n_power = 0, weight_steps = 0;
+    static constexpr int kIteratedSteps = 20;
+    void set_power(int chain, bool power) {
+        n_power += (int)power - (int)chain_power[chain];
+        chain_power[chain] = power;
+    }
+    void weights_given() { weight_steps = std::max(weight_steps, kIteratedSteps); }
 
     // host mirrors
     std::vector<eamc::TileDesc> tiles;
