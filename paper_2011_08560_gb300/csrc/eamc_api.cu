@@ -646,13 +646,14 @@ extern "C" int muca_set_eg(ea_ctx *ctx, int chain0, int n, const int32_t *e_g) {
 // slower as chains share schedulers) and one lane per chain (muca_checker.cu: 45 to 220 cycles by
 // size and tile width, the same for every chain of a block, one block per SM).  The plan estimates
 // both times of a launch, in cycles, and takes the shorter:
-//   walk:    f h (23 a_max + 10.2 sum of a / schedulers), a = attempts of a chain, f by L, fitted to
-//            512 .. 16384 chains; h: a walk moves fast while attempts are refused, as in the low energies
-//            that a power-law chain reaches after some weight steps (0.92), and slows where most are
-//            accepted, in first steps and flat ensembles (1.2; at L <= 5 no difference);
+//   walk:    f h (14.5 a_max + 10.2 sum of a / schedulers), a = attempts of a chain, f by L, fitted to
+//            1024 .. 8192 chains; h: a walk moves fast while attempts are refused, as in the low energies
+//            that a power-law chain reaches step by step (1.5 at its first weight step, 0.97 from the
+//            27th), and slower where most are accepted, as in flat ensembles (not below 1.38; no
+//            difference at L <= 5);
 //   checker: cycles(L, width) a per wave of one block per SM, as measured.
 // Both sides, attempts/ns, walk / checker.  L = 8 in tiles of 16, 4096 power-law chains after 1, 10, 20,
-// 40 weight steps 68, 81, 90, 100 / 89, flat ones 68 to 76 / 89; 2048 58 to 83 / 88; 1024 53 to 76 / 45.
+// 40 weight steps 68, 81, 90, 100 / 89, flat ones 68 to 76 / 89; 2048 58 to 83 / 88; 1024 45 to 76 / 45.
 // L = 6 in full tiles, 2048 50, 61, 66, 69 / 65, flat 50 to 57 / 65; 4096 59 to 83 / 130; 1024 47 / 33.
 // L = 10, 4096 58 to 80 / 78; 1024 39 to 55 / 21.  L = 12, 4096 61 to 82 / 70 to 80.  L = 7 in tiles of 16,
 // 2048 50 to 74 / 51.  L = 5, 4096 56 / 58; 2048 50 / 29.  L = 4, 4096 65 / 84; 2048 57 / 42.
@@ -663,17 +664,17 @@ struct ColourPlan {
 };
 
 static ColourPlan colour_plan(const ea_ctx *ctx) {
-    static const double f_walk[13] = {0, 0, 0, 4.1, 1.4, 1.6, 1.09, 1.13, 1.0, 1.15, 1.28, 1.28, 1.18};
+    static const double f_walk[13] = {0, 0, 0, 4.9, 1.55, 1.85, 1.15, 1.15, 1.0, 1.2, 1.25, 1.25, 1.18};
     static const double c_full[13] = {0, 0, 0, 220, 100, 146, 64.5, 155, 101, 125, 104, 137, 111};
     static const double c_half[13] = {0, 0, 0, 0, 79, 113, 60.5, 83, 47.5, 0, 0, 0, 0};
     ColourPlan walk, checker;
     checker.walk = false;
-    const bool low = 2 * (size_t)ctx->n_power >= ctx->chain_slot.size() && ctx->weight_steps >= ea_ctx::kIteratedSteps;
-    const double h = low ? 0.92 : 1.2;
+    const bool power = 2 * (size_t)ctx->n_power >= ctx->chain_slot.size();
+    const double h = std::max(power ? 0.97 : 1.38, 1.5 - 0.02 * std::max(0, ctx->weight_steps - 1));
     bool have = true;  // the checker kernel has every tile's width
     double w_max = 0, w_sum = 0, c_max = 0, c_sum = 0;
     for (const TileDesc &td : ctx->tiles) {
-        const double a = (double)td.V * std::max(1, td.sweep_mul), f = td.dim == 3 ? f_walk[td.L] * (td.L > 5 ? h : 1.0) : 1.5;
+        const double a = (double)td.V * std::max(1, td.sweep_mul), f = td.dim == 3 ? f_walk[td.L] * (td.L > 5 ? h : 1.0) : 1.75;
         walk.smem = std::max(walk.smem, walk_smem_bytes(td.dim, td.L));
         walk.max_width = std::max(walk.max_width, (int)td.width);
         w_max = std::max(w_max, f * a);
@@ -687,7 +688,7 @@ static ColourPlan colour_plan(const ea_ctx *ctx) {
         c_sum += c;
     }
     const double n_sm = std::max(ctx->n_sm, 1), nt = (double)ctx->tiles.size();
-    const double t_walk = 23.0 * w_max + 10.2 * w_sum / (4.0 * n_sm);
+    const double t_walk = 14.5 * w_max + 10.2 * w_sum / (4.0 * n_sm);
     const double t_checker = std::max(c_max, std::ceil(nt / n_sm) * c_sum / nt);
     return have && t_checker < t_walk ? checker : walk;
 }
