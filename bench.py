@@ -42,25 +42,23 @@ UNIT = "attempts/ns"
 # 32 chains per word with extraction 3.5, threshold fetch and compare 3, flip and energy update
 # 2, lowest energy and round-trip check 1.5); the midpoint of the scope's 25-35
 ALG_OPS_PER_ATTEMPT = 30.0
-# per-chain latency floor of one MUCA attempt in SM cycles: the next attempt's threshold is a
-# shared-memory load whose address depends on the current decision (the bin moves only if the
-# attempt is accepted), loaded for both outcomes one attempt ahead and selected.  That minimal
-# dependent pattern (select the address, load, select the threshold, compare), timed alone in one
-# warp with clock64 over 4096 steps on the GB300, takes 35.4 cycles per step (a chain of
-# dependent shared-memory loads: 34.0; compare -> select: 8.6; the same loads at independent
-# addresses pipeline at 9.2): the load's latency is not hidden once its address depends on the
-# decision it feeds, also with the loads issued two attempts ahead (32.4)
-LATENCY_FLOOR_CYCLES = 35.4
+# per-chain latency floor of one MUCA attempt in SM cycles.  The headline kernel decides 32 attempts of
+# a chain from masks made beforehand (no load depends on a decision): four segments of eight steps
+# side by side, each step shift -> and -> multiply-add, 14.8 cycles in one warp with clock64 on the
+# GB300; before them a mask load (34), after them the segments' ends through shared memory (34) and
+# four byte selects (18): 8 x 14.8 + 34 + 34 + 18 = 204 cycles per 32 attempts.  A kernel that loads a
+# threshold per attempt (the lexicographic order) cannot go below 35.4 cycles (select the address,
+# load, select the threshold, compare, timed the same way)
+LATENCY_FLOOR_CYCLES = {"colour": 6.4, "lex": 35.4}
 # PT, per site word of 32 lattices (32 attempts): 12 word loads + 14 bit ops for the
 # unsatisfied counts + 4 for the classes, about 8 compared bit planes (2 Philox4x32-10 calls of
 # 40 ops, 5 ops per plane) and the flip: about 150 lane-operations per 32 attempts
 PT_ALG_OPS = 4.7
 # dram__bytes_read.sum + dram__bytes_write.sum of one production launch of the headline workload
-# (L=8, 1024 chains in tiles of 8, checkerboard kernel), ncu capture of this kernel version:
-# 14.20 MB + 0 B for a 2000-sweep launch.  It is the one-time staging of the threshold tables and
-# lattices, so it does not grow with the sweeps of a launch: a 10^4-sweep launch moves the same
-# bytes.
-SWEEP_TRAFFIC_BYTES = 14.20e6
+# (L=8, 1024 chains, warp-per-chain kernel), ncu capture of this kernel version: 6.42 MB + 0 B for a
+# 2000-sweep launch.  It is the one-time staging of lattices and of the tables' parts around each
+# chain's bins, so it hardly grows with the sweeps of a launch.
+SWEEP_TRAFFIC_BYTES = 6.42e6
 
 
 def parse():
@@ -709,7 +707,8 @@ def build_uneven(eamc, autotune, stream_ptr, S: int, order: int = 0):
 def bench_uneven(S: int = 100, iters: int = 3, order: int = 0):
     """Uneven batch: 4096 realizations, L uniform over {4,6,8,10,12} (round robin by id), each
     as a power-law, a flat and a 1/k chain, in one launch per step (lexicographic order: the
-    persistent work-queue kernel; checkerboard order: one block per tile); the
+    persistent work-queue kernel; checkerboard order: one warp per chain, or one block
+    per tile where full tiles fill the GPU); the
     weight-iteration loop is a captured CUDA graph."""
     import torch
 
@@ -1088,7 +1087,7 @@ def main():
             torch.distributed.destroy_process_group()
         return
     attempts_e2e = r["attempts_per_step"] * world
-    lat_peak = world * r["n_chains"] * r["sm_max_mhz"] * 1e-3 / LATENCY_FLOOR_CYCLES
+    lat_peak = world * r["n_chains"] * r["sm_max_mhz"] * 1e-3 / LATENCY_FLOOR_CYCLES[W.order]
     line = {
         "metric": METRIC, "value": r["value"], "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": r["t_ms"] / args.steps, "higher_is_better": True,
@@ -1102,11 +1101,11 @@ def main():
         # round trips/s against the ALU roofline: attempts/s at the roofline / (V x mean tau)
         "round_trips_roofline": rt_roofline(r, world),
         # the bound that applies to a batch of serial chains: every chain needs at least
-        # LATENCY_FLOOR_CYCLES per attempt (select + shared-memory load + compare, loads issued
-        # one attempt ahead), so attempts/ns <= chains x SM clock / floor
+        # LATENCY_FLOOR_CYCLES per attempt (the dependent chain of its order's kernel), so
+        # attempts/ns <= chains x SM clock / floor
         "latency_roofline": {"achieved": r["value"], "peak": lat_peak, "unit": UNIT,
                              "frac": r["value"] / lat_peak,
-                             "cycles_per_attempt_floor": LATENCY_FLOOR_CYCLES,
+                             "cycles_per_attempt_floor": LATENCY_FLOOR_CYCLES[W.order],
                              "cycles_per_attempt_achieved": world * r["n_chains"] * r["sm_max_mhz"] * 1e-3 / r["value"]},
         "plain_form": r["plain"],
         "e2e": {"value": attempts_e2e / (r["e2e_ms"] * 1e6), "unit": UNIT,
@@ -1118,7 +1117,7 @@ def main():
                      "frac": r["achieved_ops"] / r["alu_peak"], "traffic": SWEEP_TRAFFIC_BYTES,
                      "traffic_basis": "ncu dram read+write of one launch (one-time table and lattice "
                                       "staging, independent of the sweeps per launch)",
-                     "kernel": "muca_checker_kernel<3, 0>" if W.order == "colour" else "muca_sweep_kernel<3>",
+                     "kernel": "muca_walk_kernel<3>" if W.order == "colour" else "muca_sweep_kernel<3>",
                      "ops_per_attempt": ALG_OPS_PER_ATTEMPT,
                      "peak_basis": f"{r['sm_count']} SMs x 128 lane-instructions/clk x max SM clock "
                                    f"(MEASURED_PEAKS.json sm_max_mhz)"},

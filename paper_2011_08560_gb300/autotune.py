@@ -10,8 +10,8 @@ Knobs:
     persistent grid (chains are latency-bound, so tiles sharing an SM sub-partition slow each
     other down);
   * sweeps per launch.
-In the colour order (muca_set_sweep_order) the even-L chains run in their own kernel, one block
-per tile: there only the tile width is tuned.  The order itself is the caller's choice (it changes
+In the colour order (muca_set_sweep_order) only the tile width is tuned; it decides little there, since
+a chain has a warp of its own unless the batch fills the GPU with full tiles.  The order itself is the caller's choice (it changes
 the trajectories), never the tuner's.
 A candidate is timed with CUDA events on a scratch context with the same composition of chains
 (same dim, L and chain counts, a different seed), so tuning never advances the caller's chains,
