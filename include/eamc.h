@@ -313,6 +313,12 @@ typedef struct {
 int pt_init(ea_ctx *ctx, int dim, int L, int n_real, uint32_t rid0, int M, const double *betas,
             const int8_t *couplings_or_null);
 
+/* a6 -- how n_real realizations at M temperatures are split on a GPU of n_sm SMs (no GPU needed): CTAs
+ * per group of 32 realizations (*ctas), temperature slots per CTA (*slots; with M no multiple the last
+ * CTA has fewer) and the shared memory a CTA needs at least (*smem_bytes).  Each may be NULL.  Results
+ * do not depend on the split.  EA_EINVAL for a dim, L, n_real or M that pt_init refuses. */
+int pt_get_split(int dim, int L, int n_real, int M, int n_sm, int *ctas, int *slots, size_t *smem_bytes);
+
 /* Round-trip bounds per realization (host int32[n_real] each): bottom E_g, top E_hot. */
 int pt_set_rt_bounds(ea_ctx *ctx, const int32_t *e_g, const int32_t *e_hot);
 

@@ -723,16 +723,20 @@ cudaError_t pt_dispatch(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, uin
     return cudaErrorInvalidValue;
 }
 
-// passes over its slots that a CTA of spc slots makes in a colour
-int pt_passes(int dim, int L, int spc) {
+// what a CTA of spc slots takes: passes over them in a colour, and shared memory (the narrow form)
+struct PtForm {
+    int passes = 0;
+    size_t smem = 0;
+};
+PtForm pt_form(int dim, int L, int spc) {
 #define PT_CASE(D, LL) \
-    if (dim == D && L == LL) return (spc + PtGeo<D, LL>::kt(spc) - 1) / PtGeo<D, LL>::kt(spc);
+    if (dim == D && L == LL) return {(spc + PtGeo<D, LL>::kt(spc) - 1) / PtGeo<D, LL>::kt(spc), PtGeo<D, LL>::smem(spc)};
     PT_CASE(3, 3) PT_CASE(3, 4) PT_CASE(3, 5) PT_CASE(3, 6) PT_CASE(3, 7) PT_CASE(3, 8) PT_CASE(3, 9)
     PT_CASE(3, 10) PT_CASE(3, 11) PT_CASE(3, 12)
     PT_CASE(2, 3) PT_CASE(2, 4) PT_CASE(2, 5) PT_CASE(2, 6) PT_CASE(2, 7) PT_CASE(2, 8) PT_CASE(2, 9)
     PT_CASE(2, 10) PT_CASE(2, 11) PT_CASE(2, 12)
 #undef PT_CASE
-    return spc;
+    return {};
 }
 
 // CTAs per realization group, at most 8 (clusters of 16 measured slower): the largest number that divides
@@ -741,14 +745,16 @@ int pt_passes(int dim, int L, int spc) {
 // blocks cost it up to that.  us per sweep, dividing -> fewest: M = 17, L = 7, 256 realizations 23.7 -> 7.9;
 // L = 8, 1024 28.7 -> 8.8; L = 12, 256 104 -> 18; L = 4, 1024 6.0 -> 3.7; M = 20, L = 10, 256 13.7 -> 10.8;
 // M = 13, L = 8, 600 21.0 -> 6.8.  Left dividing: M = 17, L = 4, 8192 9.5 (11.2); M = 20, L = 6, 1024 6.8
-// (7.5), L = 8, 2048 16.6 (17.4).
+// (7.5), L = 8, 2048 16.6 (17.4).  A dividing split whose slots exceed a block's shared memory (a prime M
+// of the larger lattices keeps them all in one block) is none; the fewest slots, 8 at most, always fit.
 int pt_cluster(int dim, int L, int M, int n_groups, int n_sm) {
     int even = 1;
     for (int c = 8; c >= 2 && even == 1; --c)
         if (M % c == 0) even = c;
     const int spc = (M + 7) / 8, least = (M + spc - 1) / spc;
+    if (pt_form(dim, L, M / even).smem > kPtSmemMax) return least;
     auto cost = [&](int cs) {
-        return (long long)pt_passes(dim, L, (M + cs - 1) / cs) * std::max((long long)n_sm, (long long)n_groups * cs);
+        return (long long)pt_form(dim, L, (M + cs - 1) / cs).passes * std::max((long long)n_sm, (long long)n_groups * cs);
     };
     return 4 * cost(even) >= 5 * cost(least) ? least : even;
 }
@@ -855,6 +861,16 @@ static int pt_upload_betas(ea_ctx *ctx, const double *betas) {
     pt_planes_kernel<<<(int)(G * M), 32, 0, ctx->stream>>>(p->d_beta, p->dim, p->d_planes);
     PT_CUDA(cudaGetLastError());
     PT_CUDA(cudaStreamSynchronize(ctx->stream));
+    return EA_OK;
+}
+
+extern "C" int pt_get_split(int dim, int L, int n_real, int M, int n_sm, int *ctas, int *slots, size_t *smem_bytes) {
+    if ((dim != 2 && dim != 3) || L < 3 || L > 12 || n_real <= 0 || M < 2 || M > 64 || n_sm <= 0)
+        return fail(EA_EINVAL, "no parallel tempering of dim=%d, L=%d, %d realizations, M=%d", dim, L, n_real, M);
+    const int cs = pt_cluster(dim, L, M, (n_real + 31) / 32, n_sm), spc = (M + cs - 1) / cs;
+    if (ctas) *ctas = cs;
+    if (slots) *slots = spc;
+    if (smem_bytes) *smem_bytes = pt_form(dim, L, spc).smem;
     return EA_OK;
 }
 

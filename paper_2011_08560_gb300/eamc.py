@@ -148,6 +148,7 @@ SIGNATURES = {
     "ea_srv_context": (_i, [P, ctypes.POINTER(P)]),
     "ea_srv_tile_bytes": (ctypes.c_size_t, [_i, _i]),
     "pt_init": (_i, [P, _i, _i, _i, _u32, _i, P, P]),
+    "pt_get_split": (_i, [_i, _i, _i, _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_i), ctypes.POINTER(ctypes.c_size_t)]),
     "pt_set_rt_bounds": (_i, [P, P, P]),
     "pt_run": (_i, [P, _u64, _i]),
     "pt_get_state": (_i, [P, P, P, P, P]),
@@ -196,6 +197,14 @@ def narrow_width(dim: int, L: int, order: int = 0) -> int:
     no narrow one)."""
     ws = narrow_widths(dim, L, order)
     return ws[0] if ws else 32
+
+
+def pt_split(dim: int, L: int, n: int, M: int, n_sm: int):
+    """(CTAs per group of 32 realizations, temperature slots per CTA, shared memory per CTA) of a
+    parallel-tempering batch on a GPU of n_sm SMs."""
+    ctas, slots, smem = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_size_t(0)
+    check(lib().pt_get_split(dim, L, n, M, n_sm, ctypes.byref(ctas), ctypes.byref(slots), ctypes.byref(smem)))
+    return ctas.value, slots.value, smem.value
 
 
 def check(rc: int) -> int:
