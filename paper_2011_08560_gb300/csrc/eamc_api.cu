@@ -852,9 +852,9 @@ extern "C" int ea_graph_capture(ea_ctx *ctx, int n_iter, uint64_t sweeps_per_ite
     if (ctx->graph) { cudaGraphDestroy(ctx->graph); ctx->graph = nullptr; }
     EA_CUDA(cudaStreamSynchronize(ctx->stream));
     // attributes are set outside the capture (they are not stream work)
-    EA_CUDA(prepare_sweeps(ctx->dim, ctx->sweep_smem));
+    EA_CUDA(prepare_sweeps(ctx->dim));
     const PartsPlan parts = parts_plan(ctx);
-    if (parts.cls >= 0) EA_CUDA(prepare_parts(parts.cls, parts.smem));
+    if (parts.cls >= 0) EA_CUDA(prepare_parts(parts.cls));
     EA_CUDA(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
     int rc = EA_OK;
     const int nt = (int)ctx->tiles.size();

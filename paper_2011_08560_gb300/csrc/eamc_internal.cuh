@@ -21,6 +21,13 @@ namespace eamc {
 constexpr uint32_t kAlways = 0xFFFFFFFFu;
 constexpr int kTile = 32;
 constexpr int kNoBottom = -1;  // b_g when no E_g is known yet: never reached
+// The dynamic shared memory that a block may ask for: all of the 227 KB, and in the sweep kernels 225 KB
+// (their threshold tables stay in global memory beyond it; the rest is static shared memory).  A kernel's
+// limit holds for every host thread that uses the device, so it is set to this one value before each launch
+// (0.2 to 0.5 us) instead of to the launch's own: no thread lowers it under another's launch, and no record
+// of what has been set has to be right for every device.
+constexpr size_t kBlockSmemMax = 227u << 10;
+constexpr size_t kSweepSmemMax = 225u << 10;
 
 struct TileDesc {
     int32_t dim, L, V, B;  // B = table rows per chain = largest b_top + 1 for this (dim, L)
@@ -111,7 +118,7 @@ int sweep_blocks_per_sm(int dim, size_t smem);
 int sweep_part_class(int L);
 int sweep_part_chains(int L);
 size_t sweep_part_smem_bytes(int L);
-cudaError_t prepare_parts(int cls, size_t smem);
+cudaError_t prepare_parts(int cls);
 cudaError_t launch_sweeps_parts(const TileDesc *d_tiles, int n_tiles, int cls, int n_parts, size_t smem,
                                 SlotState *d_slots, uint32_t *d_spins, const uint32_t *d_bonds, const uint32_t *d_thr,
                                 uint32_t *d_hist, uint64_t n_sweeps, PhiloxKey key, int count_rt, unsigned *d_diag,
@@ -134,7 +141,7 @@ cudaError_t launch_sweeps_checker(const TileDesc *d_tiles, int n_tiles, int dim,
                                   uint32_t *d_spins, const uint32_t *d_bonds, const uint32_t *d_thr,
                                   uint32_t *d_hist, uint64_t n_sweeps, PhiloxKey key, int count_rt,
                                   unsigned *d_diag, cudaStream_t st, int parities);
-cudaError_t prepare_sweeps(int dim, size_t smem);  // resident sweep blocks per SM at this smem
+cudaError_t prepare_sweeps(int dim);
 cudaError_t launch_quantize(const TileDesc *d_tiles, int n_tiles, const SlotState *d_slots,
                             const double *d_lnW, uint32_t *d_thr, cudaStream_t st);
 cudaError_t launch_quantize_selected(const TileDesc *d_tiles, int n_tiles, const SlotState *d_slots,

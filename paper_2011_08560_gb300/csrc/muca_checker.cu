@@ -128,7 +128,7 @@ struct CkGeo {
     static constexpr int NPR = NP * RPR;
     static constexpr size_t FSH_BYTES = (L & 1) ? ((size_t)2 * NCOL * NPR * 4 + 15) / 16 * 16 : 0;
     static constexpr size_t BASE_BYTES = LATTICE_BYTES + HAND_BYTES + RES_BYTES + FSH_BYTES;
-    static constexpr bool SMEM_THR = BASE_BYTES + THR_BYTES <= 225 * 1024;
+    static constexpr bool SMEM_THR = BASE_BYTES + THR_BYTES <= kSweepSmemMax;
     static constexpr size_t SMEM = BASE_BYTES + (SMEM_THR ? THR_BYTES : 0);
     // thresholds addressed by 32-bit shared addresses; measured with the same launches: L = 6 in
     // tiles of 32 2.5 % faster, L = 8 in tiles of 16 2.5 % slower
@@ -613,13 +613,9 @@ template <int DIM, int MODE>
 cudaError_t ck_launch(int n_tiles, size_t smem, cudaStream_t st, const TileDesc *d_tiles, SlotState *d_slots,
                       uint32_t *d_spins, const uint32_t *d_bonds, const uint32_t *d_thr, uint32_t *d_hist,
                       uint64_t n_sweeps, PhiloxKey key, int count_rt, unsigned *d_diag) {
-    static size_t set_limit = 0;
-    if (smem > set_limit) {
-        const cudaError_t e = cudaFuncSetAttribute(muca_checker_kernel<DIM, MODE>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        set_limit = smem;
-    }
+    const cudaError_t e = cudaFuncSetAttribute(muca_checker_kernel<DIM, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kSweepSmemMax);
+    if (e != cudaSuccess) return e;
     muca_checker_kernel<DIM, MODE><<<n_tiles, kCkThreads, smem, st>>>(d_tiles, d_slots, d_spins, d_bonds, d_thr,
                                                                        d_hist, n_sweeps, key, count_rt, d_diag);
     return cudaGetLastError();

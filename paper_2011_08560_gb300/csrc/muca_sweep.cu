@@ -98,8 +98,7 @@ struct Geo {
     static constexpr size_t RES_BYTES = (size_t)2 * L * W * sizeof(int);  // row offsets, measurement
     static constexpr size_t THR_BYTES = (size_t)(B + 2 * DIM) * 8 * W * sizeof(uint32_t);
     static constexpr size_t BASE_BYTES = LATTICE_BYTES + HAND_BYTES + RES_BYTES;
-    // up to 225 KB of the 227 KB a block may use (the rest: static shared memory)
-    static constexpr bool SMEM_THR = BASE_BYTES + THR_BYTES <= 225 * 1024;
+    static constexpr bool SMEM_THR = BASE_BYTES + THR_BYTES <= kSweepSmemMax;
     static constexpr size_t SMEM = BASE_BYTES + (SMEM_THR ? THR_BYTES : 0);
 };
 
@@ -646,16 +645,11 @@ bool sweep_thresholds_in_smem(int dim, int L, int width) {
     return thr_smem_w<2, 32>(L);
 }
 
-// Raises the kernel's dynamic shared-memory limit when needed (a host call that is not stream
-// work, so it happens before any graph capture that launches the kernel).
-cudaError_t prepare_sweeps(int dim, size_t smem) {
-    static int set_limit[4] = {0, 0, 0, 0};
-    if ((int)smem <= set_limit[dim]) return cudaSuccess;
-    const cudaError_t e = dim == 3
-        ? cudaFuncSetAttribute(muca_sweep_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-        : cudaFuncSetAttribute(muca_sweep_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) set_limit[dim] = (int)smem;
-    return e;
+// Raises the kernel's dynamic shared-memory limit (a host call that is not stream work, so it
+// happens before any graph capture that launches the kernel).
+cudaError_t prepare_sweeps(int dim) {
+    const void *k = dim == 3 ? (const void *)muca_sweep_kernel<3> : (const void *)muca_sweep_kernel<2>;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmemMax);
 }
 
 cudaError_t launch_sweeps(const TileDesc *d_tiles, const int32_t *d_tile_list, int n_blocks, int n_work,
@@ -668,7 +662,7 @@ cudaError_t launch_sweeps(const TileDesc *d_tiles, const int32_t *d_tile_list, i
         e = cudaMemsetAsync(d_queue, 0, sizeof(int), st);
         if (e != cudaSuccess) return e;
     }
-    if ((e = prepare_sweeps(dim, smem)) != cudaSuccess) return e;
+    if ((e = prepare_sweeps(dim)) != cudaSuccess) return e;
     if (dim == 3) {
         muca_sweep_kernel<3><<<n_blocks, kThreads, smem, st>>>(d_tiles, d_tile_list, n_work, d_queue, d_slots, d_spins,
                                                          d_bonds, d_thr, d_hist, n_sweeps, key, count_rt, d_diag);
@@ -693,12 +687,8 @@ static const void *parts_kernel(int cls) {
     return k[cls];
 }
 
-cudaError_t prepare_parts(int cls, size_t smem) {
-    static size_t set_limit[3] = {0, 0, 0};
-    if (smem <= set_limit[cls]) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(parts_kernel(cls), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) set_limit[cls] = smem;
-    return e;
+cudaError_t prepare_parts(int cls) {
+    return cudaFuncSetAttribute(parts_kernel(cls), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmemMax);
 }
 
 cudaError_t launch_sweeps_parts(const TileDesc *d_tiles, int n_tiles, int cls, int n_parts, size_t smem,
@@ -706,7 +696,7 @@ cudaError_t launch_sweeps_parts(const TileDesc *d_tiles, int n_tiles, int cls, i
                                 uint32_t *d_hist, uint64_t n_sweeps, PhiloxKey key, int count_rt, unsigned *d_diag,
                                 cudaStream_t st) {
     if (n_tiles <= 0 || n_sweeps == 0) return cudaSuccess;
-    const cudaError_t e = prepare_parts(cls, smem);
+    const cudaError_t e = prepare_parts(cls);
     if (e != cudaSuccess) return e;
     const int grid = n_tiles * n_parts;
 #define EAMC_PARTS(C) \

@@ -102,7 +102,6 @@ __device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
 }
 
 constexpr int kTailQ = 32;  // open comparisons a warp defers per colour phase
-constexpr size_t kPtSmemMax = 227u << 10;  // shared memory of a block
 
 template <int DIM, int L, bool WIDE = false>
 struct PtGeo {
@@ -647,7 +646,7 @@ cudaError_t pt_launch_sweeps(const PtState *p, const PtArgs &a, cudaStream_t st)
     using G = PtGeo<DIM, L, WIDE>;
     const int threads = G::threads(a.spc);
     const size_t smem = G::smem(a.spc);
-    cudaError_t e = cudaFuncSetAttribute(pt_kernel<DIM, L, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(pt_kernel<DIM, L, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlockSmemMax);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(pt_kernel<DIM, L, WIDE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
@@ -706,7 +705,7 @@ cudaError_t pt_launch_all(PtState *p, const int8_t *dJ, ea_ctx *ctx, int what, u
     if constexpr (DIM == 3 && L >= 8) {
         using W = PtGeo<DIM, L, true>;
         if (4 * p->n_groups * p->cs <= 3 * ctx->n_sm && W::threads(a.spc) > G::threads(a.spc) &&
-            W::smem(a.spc) <= kPtSmemMax)
+            W::smem(a.spc) <= kBlockSmemMax)
             return pt_launch_sweeps<DIM, L, true>(p, a, ctx->stream);
     }
     return pt_launch_sweeps<DIM, L, false>(p, a, ctx->stream);
@@ -752,7 +751,7 @@ int pt_cluster(int dim, int L, int M, int n_groups, int n_sm) {
     for (int c = 8; c >= 2 && even == 1; --c)
         if (M % c == 0) even = c;
     const int spc = (M + 7) / 8, least = (M + spc - 1) / spc;
-    if (pt_form(dim, L, M / even).smem > kPtSmemMax) return least;
+    if (pt_form(dim, L, M / even).smem > kBlockSmemMax) return least;
     auto cost = [&](int cs) {
         return (long long)pt_form(dim, L, (M + cs - 1) / cs).passes * std::max((long long)n_sm, (long long)n_groups * cs);
     };
