@@ -165,6 +165,17 @@ int muca_set_launch(ea_ctx *ctx, int persistent, uint64_t sweeps_per_launch, int
  * of a snapshot.  EA_EINVAL for an unknown order or count. */
 int muca_set_sweep_order(ea_ctx *ctx, int order, int chains_per_cta);
 
+/* a2 -- the kernel that runs the colour order in this context: EA_COLOUR_AUTO (the default) takes the
+ * one that the library estimates to be faster; EA_COLOUR_WARP is one warp per chain, EA_COLOUR_LANE
+ * one lane per chain.  Results do not depend on it.  EA_COLOUR_LANE runs full tiles and, in 3D, tiles
+ * of 16 at L = 4..8; with narrower ones muca_run_sweeps and ea_graph_capture then refuse (EA_EINVAL).
+ * muca_get_colour_kernel: the kernel that the next muca_run_sweeps in the colour order takes. */
+#define EA_COLOUR_AUTO 0
+#define EA_COLOUR_WARP 1
+#define EA_COLOUR_LANE 2
+int muca_set_colour_kernel(ea_ctx *ctx, int kernel);
+int muca_get_colour_kernel(ea_ctx *ctx, int *kernel);
+
 /* a8 -- chains per tile for chains of linear size L added afterwards (ea_init_disorder):
  * width 32 (the default, every L), 16 (3D, L = 7, 8), or, for chains swept in the colour order
  * only, 16 (3D, L = 4, 5, 6), 8 (3D, L = 4..10) and 4 (3D, L = 11, 12); muca_run_sweeps in the

@@ -658,7 +658,7 @@ extern "C" int muca_set_eg(ea_ctx *ctx, int chain0, int n, const int32_t *e_g) {
 // L = 10, 4096 58 to 80 / 78; 1024 39 to 55 / 21.  L = 12, 4096 61 to 82 / 70 to 80.  L = 7 in tiles of 16,
 // 2048 50 to 74 / 51.  L = 5, 4096 56 / 58; 2048 50 / 29.  L = 4, 4096 65 / 84; 2048 57 / 42.
 struct ColourPlan {
-    bool walk = true;
+    bool walk = true, runs = true;  // runs: the kernel has every tile's width
     size_t smem = 0;
     int max_width = 0, parities = 0;
 };
@@ -690,6 +690,9 @@ static ColourPlan colour_plan(const ea_ctx *ctx) {
     const double n_sm = std::max(ctx->n_sm, 1), nt = (double)ctx->tiles.size();
     const double t_walk = 14.5 * w_max + 10.2 * w_sum / (4.0 * n_sm);
     const double t_checker = std::max(c_max, std::ceil(nt / n_sm) * c_sum / nt);
+    checker.runs = have;
+    if (ctx->colour_kernel == EA_COLOUR_WARP) return walk;
+    if (ctx->colour_kernel == EA_COLOUR_LANE) return checker;
     return have && t_checker < t_walk ? checker : walk;
 }
 
@@ -725,6 +728,7 @@ int ctx_enqueue_sweeps(ea_ctx *ctx, uint64_t n_sweeps, int count_roundtrips) {
     const uint64_t chunk = ctx->sweeps_per_launch ? ctx->sweeps_per_launch : n_sweeps;
     if (ctx->order == 1) {
         const ColourPlan plan = colour_plan(ctx);
+        if (!plan.runs) return fail(EA_EINVAL, "tiles of this context run only with a warp per chain");
         unsigned *diag = reinterpret_cast<unsigned *>(ctx->d_queue + 1);
         for (uint64_t done = 0; done < n_sweeps; done += chunk) {
             const uint64_t now = std::min(chunk, n_sweeps - done);
@@ -803,7 +807,22 @@ extern "C" int muca_set_sweep_order(ea_ctx *ctx, int order, int chains_per_cta) 
     if (chains_per_cta != 0 && (chains_per_cta < 1 || chains_per_cta > 8 || (32 % chains_per_cta) != 0))
         return fail(EA_EINVAL, "chains_per_cta must be 0 or one of 1, 2, 4, 8");
     ctx->order = order;
-    (void)chains_per_cta;  // no effect: the colour order runs one lane per chain at every L
+    (void)chains_per_cta;  // no effect
+    return EA_OK;
+}
+
+extern "C" int muca_set_colour_kernel(ea_ctx *ctx, int kernel) {
+    if (!ctx) return fail(EA_EINVAL, "null context");
+    if (kernel != EA_COLOUR_AUTO && kernel != EA_COLOUR_WARP && kernel != EA_COLOUR_LANE)
+        return fail(EA_EINVAL, "unknown colour-order kernel %d", kernel);
+    ctx->colour_kernel = kernel;
+    return EA_OK;
+}
+
+extern "C" int muca_get_colour_kernel(ea_ctx *ctx, int *kernel) {
+    if (!ctx || !kernel) return fail(EA_EINVAL, "null argument");
+    if (ctx->tiles.empty()) return fail(EA_ESTATE, "no chains: call ea_init_disorder first");
+    *kernel = colour_plan(ctx).walk ? EA_COLOUR_WARP : EA_COLOUR_LANE;
     return EA_OK;
 }
 

@@ -19,6 +19,7 @@ EA_ALWAYS = 0xFFFFFFFF
 EA_FLAT, EA_POWERLAW, EA_ONE_OVER_K, EA_CANON = 0, 1, 2, 3
 EA_REC_PLAIN, EA_REC_BERG = 0, 1
 EA_ORDER_LEX, EA_ORDER_COLOUR = 0, 1
+EA_COLOUR_AUTO, EA_COLOUR_WARP, EA_COLOUR_LANE = 0, 1, 2
 
 
 class EamcError(RuntimeError):
@@ -130,6 +131,8 @@ SIGNATURES = {
     "muca_set_sweep_multiplier": (_i, [P, _i, _i]),
     "muca_set_tile_width": (_i, [P, _i, _i]),
     "muca_set_sweep_order": (_i, [P, _i, _i]),
+    "muca_set_colour_kernel": (_i, [P, _i]),
+    "muca_get_colour_kernel": (_i, [P, ctypes.POINTER(_i)]),
     "muca_get_tile_width": (_i, [_i, _i, _i, ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(_i)]),
     "muca_get_tile_width_colour": (_i, [_i, _i, _i, ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(_i)]),
     "muca_update_weights_subset": (_i, [P, P, _i]),
@@ -400,6 +403,16 @@ class Context:
     def set_sweep_order(self, order: int, chains_per_cta: int = 0):
         """EA_ORDER_LEX or EA_ORDER_COLOUR for every chain of the context (see the header)."""
         check(lib().muca_set_sweep_order(self._h, order, chains_per_cta))
+
+    def set_colour_kernel(self, kernel: int):
+        """The colour order's kernel: EA_COLOUR_AUTO, EA_COLOUR_WARP or EA_COLOUR_LANE (see the header)."""
+        check(lib().muca_set_colour_kernel(self._h, kernel))
+
+    def colour_kernel(self) -> int:
+        """The kernel that the next sweeps in the colour order take: EA_COLOUR_WARP or EA_COLOUR_LANE."""
+        kernel = ctypes.c_int(0)
+        check(lib().muca_get_colour_kernel(self._h, ctypes.byref(kernel)))
+        return kernel.value
 
     def set_tile_width(self, L: int, width: int):
         """Chains per tile (32, or 16 for L = 7, 8 in 3D) for chains of size L added
