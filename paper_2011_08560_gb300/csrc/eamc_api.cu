@@ -641,40 +641,55 @@ extern "C" int muca_set_eg(ea_ctx *ctx, int chain0, int n, const int32_t *e_g) {
     return EA_OK;
 }
 
-// The colour order has two kernels with the same results: one warp per chain (muca_walk.cu: 22 cycles
-// per attempt of a chain that has a scheduler to itself, and about 11 issue cycles per attempt, so
-// slower as chains share schedulers) and one lane per chain (muca_checker.cu: 45 to 220 cycles by
-// size and tile width, the same for every chain of a block, one block per SM).  The plan estimates
-// both times of a launch, in cycles, and takes the shorter:
-//   walk:    f h (14.5 a_max + 10.2 sum of a / schedulers), a = attempts of a chain, f by L, fitted to
-//            1024 .. 8192 chains; h: a walk moves fast while attempts are refused, as in the low energies
-//            that a power-law chain reaches step by step (1.5 at its first weight step, 0.97 from the
-//            27th), and slower where most are accepted, as in flat ensembles (not below 1.38; no
-//            difference at L <= 5);
-//   checker: cycles(L, width) a per wave of one block per SM, as measured.
-// Both sides, attempts/ns, walk / checker.  L = 8 in tiles of 16, 4096 power-law chains after 1, 10, 20,
-// 40 weight steps 68, 81, 90, 100 / 89, flat ones 68 to 76 / 89; 2048 58 to 83 / 88; 1024 45 to 76 / 45.
-// L = 6 in full tiles, 2048 50, 61, 66, 69 / 65, flat 50 to 57 / 65; 4096 59 to 83 / 130; 1024 47 / 33.
-// L = 10, 4096 58 to 80 / 78; 1024 39 to 55 / 21.  L = 12, 4096 61 to 82 / 70 to 80.  L = 7 in tiles of 16,
-// 2048 50 to 74 / 51.  L = 5, 4096 56 / 58; 2048 50 / 29.  L = 4, 4096 65 / 84; 2048 57 / 42.
+// The colour order has two kernels with the same results: one warp per chain (muca_walk.cu: 26 cycles
+// per attempt of a chain that has a scheduler to itself, slower as chains share schedulers) and one
+// lane per chain (muca_checker.cu: 45 to 300 cycles by size and tile width, the same for every chain of
+// a block, one block per SM).  The plan estimates both times of a launch, in cycles, and takes the shorter.
+//   walk:    a (f / r) T(q).  a: attempts of a chain.  q: chains per scheduler; T: cycles that q chains
+//            of L = 8 take at f = 1 (four at most are resident on a scheduler).  f by dim and L, for
+//            chains that accept most attempts, as with constant weights.  r = 1 + g ln(1 + s / 6) after s
+//            weight steps: a walk moves faster the more attempts are refused, as in the low energies that
+//            a power-law chain reaches step by step; flat ensembles gain a third of that.  L = 8, 2048
+//            power-law chains after 0, 1, 5, 10, 20, 40 steps of 300 sweeps: r = 1, 1.06, 1.19, 1.32, 1.49,
+//            1.69 (estimate 1, 1.05, 1.20, 1.33, 1.49, 1.68), flat ones 1.18 after 40.
+//   checker: cycles(dim, L, width) a per wave of one block per SM, as measured.
+// The estimate of the walk kernel is within 10 % over 600 to 9728 chains, L = 3..12 in 2D and 3D.  Both
+// sides measured, attempts/ns, walk / checker.  L = 8 in tiles of 16, power law, 4096 chains after 1, 10, 20,
+// 40 weight steps 68, 81, 90, 100 / 89; 2432 after 1 step 70 / 105; 1024 45 to 76 / 45.  L = 6 in full tiles, 2048
+// 50, 61, 66, 69 / 65; 4096 59 to 83 / 130; 1024 47 / 33.  L = 7, full, 4864 62 to 86 / 65; L = 9, 63 to 83 / 70;
+// L = 11, 61 to 76 / 65 to 73; L = 10, 4096 58 to 80 / 78; L = 5, 4864 50 to 60 / 68; L = 4, 4096 65 / 84; L = 3, 2432
+// 20 / 23.  2D: L = 3, 1024 4.3 / 7.0; L = 4, 1024 12 / 19, 2048 16 / 37; L = 5, 512 6.6 / 6.3, 1024 11 / 13; L = 8, 1024
+// 40 / 32, 1536 50 / 49, 2048 53 / 65; L = 12, 1024 40 / 32, 1536 49 / 48, 2048 52 / 64 (after 27 steps 2432 72 / 76).
 struct ColourPlan {
     bool walk = true, runs = true;  // runs: the kernel has every tile's width
     size_t smem = 0;
     int max_width = 0, parities = 0;
 };
 
+// cycles per attempt (f = 1) of q chains to a scheduler: rounds of four, then the rest
+static double walk_cycles(double q) {
+    q -= 1e-9;  // whole numbers out of sums
+    const double full = std::max(0.0, std::ceil(q / 4) - 1);
+    return 44 * full + std::max(26.0, 14.4 + 8.65 * std::ceil(q - 4 * full));
+}
+
 static ColourPlan colour_plan(const ea_ctx *ctx) {
-    static const double f_walk[13] = {0, 0, 0, 4.9, 1.55, 1.85, 1.15, 1.15, 1.0, 1.2, 1.25, 1.25, 1.18};
-    static const double c_full[13] = {0, 0, 0, 220, 100, 146, 64.5, 155, 101, 125, 104, 137, 111};
-    static const double c_half[13] = {0, 0, 0, 0, 79, 113, 60.5, 83, 47.5, 0, 0, 0, 0};
+    static const double f_3d[13] = {0, 0, 0, 5.15, 1.8, 2.15, 1.75, 1.77, 1.56, 1.72, 1.84, 1.84, 1.77};
+    static const double g_3d[13] = {0, 0, 0, 0.01, 0.09, 0.14, 0.24, 0.26, 0.335, 0.25, 0.25, 0.2, 0.23};
+    static const double f_2d[13] = {0, 0, 0, 15, 5.7, 5.9, 2.75, 3.15, 1.65, 2.1, 1.82, 2.12, 1.65};
+    static const double c_full[13] = {0, 0, 0, 222, 100, 147, 64.5, 157, 101, 137, 104, 143, 111};
+    static const double c_half[13] = {0, 0, 0, 0, 78, 114, 60.5, 83, 47.5, 0, 0, 0, 0};
+    static const double c_2d[13] = {0, 0, 0, 303, 114, 168, 101, 128, 65.5, 99, 78.5, 89.4, 66};
     ColourPlan walk, checker;
     checker.walk = false;
     const bool power = 2 * (size_t)ctx->n_power >= ctx->chain_slot.size();
-    const double h = std::max(power ? 0.97 : 1.38, 1.5 - 0.02 * std::max(0, ctx->weight_steps - 1));
+    const double steps = std::log(1 + ctx->weight_steps / 6.0) * (power ? 1.0 : 1.0 / 3);
     bool have = true;  // the checker kernel has every tile's width
     double w_max = 0, w_sum = 0, c_max = 0, c_sum = 0;
     for (const TileDesc &td : ctx->tiles) {
-        const double a = (double)td.V * std::max(1, td.sweep_mul), f = td.dim == 3 ? f_walk[td.L] * (td.L > 5 ? h : 1.0) : 1.75;
+        const double a = (double)td.V * std::max(1, td.sweep_mul);
+        const double g = td.dim == 3 ? g_3d[td.L] : std::max(0.0, 0.02 * td.L - 0.11);
+        const double f = (td.dim == 3 ? f_3d[td.L] : f_2d[td.L]) / (1 + g * steps);
         walk.smem = std::max(walk.smem, walk_smem_bytes(td.dim, td.L));
         walk.max_width = std::max(walk.max_width, (int)td.width);
         w_max = std::max(w_max, f * a);
@@ -683,12 +698,12 @@ static ColourPlan colour_plan(const ea_ctx *ctx) {
         have = have && ck > 0;
         checker.smem = std::max(checker.smem, ck);
         checker.parities |= checker_parity_class(td.dim, td.L, td.width);
-        const double c = a * (td.dim == 3 ? (td.width == 32 ? c_full[td.L] : c_half[td.L]) : 100.0);
+        const double c = a * (td.dim == 2 ? c_2d[td.L] : td.width == 32 ? c_full[td.L] : c_half[td.L]);
         c_max = std::max(c_max, c);
         c_sum += c;
     }
     const double n_sm = std::max(ctx->n_sm, 1), nt = (double)ctx->tiles.size();
-    const double t_walk = 14.5 * w_max + 10.2 * w_sum / (4.0 * n_sm);
+    const double t_walk = w_max * walk_cycles(w_sum / w_max / (4.0 * n_sm));  // chains of the longest's length
     const double t_checker = std::max(c_max, std::ceil(nt / n_sm) * c_sum / nt);
     checker.runs = have;
     if (ctx->colour_kernel == EA_COLOUR_WARP) return walk;

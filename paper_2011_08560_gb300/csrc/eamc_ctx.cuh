@@ -24,7 +24,7 @@ struct ea_ctx {
     // steps since the newest chains were made, given weights counted as kIteratedSteps of them
     std::vector<uint8_t> chain_power;
     int n_power = 0, weight_steps = 0;
-    static constexpr int kIteratedSteps = 27;
+    static constexpr int kIteratedSteps = 40;
     void set_power(int chain, bool power) {
         n_power += (int)power - (int)chain_power[chain];
         chain_power[chain] = power;
