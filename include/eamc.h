@@ -167,8 +167,7 @@ int muca_set_sweep_order(ea_ctx *ctx, int order, int chains_per_cta);
 
 /* a2 -- the kernel that runs the colour order in this context: EA_COLOUR_AUTO (the default) takes the
  * one that the library estimates to be faster; EA_COLOUR_WARP is one warp per chain, EA_COLOUR_LANE
- * one lane per chain.  Results do not depend on it.  EA_COLOUR_LANE runs full tiles and, in 3D, tiles
- * of 16 at L = 4..8; with narrower ones muca_run_sweeps and ea_graph_capture then refuse (EA_EINVAL).
+ * one lane per chain.  Results do not depend on it.
  * muca_get_colour_kernel: the kernel that the next muca_run_sweeps in the colour order takes. */
 #define EA_COLOUR_AUTO 0
 #define EA_COLOUR_WARP 1

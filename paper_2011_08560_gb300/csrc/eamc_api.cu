@@ -7,6 +7,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -652,7 +653,18 @@ extern "C" int muca_set_eg(ea_ctx *ctx, int chain0, int n, const int32_t *e_g) {
 //            a power-law chain reaches step by step; flat ensembles gain a third of that.  L = 8, 2048
 //            power-law chains after 0, 1, 5, 10, 20, 40 steps of 300 sweeps: r = 1, 1.06, 1.19, 1.32, 1.49,
 //            1.69 (estimate 1, 1.05, 1.20, 1.33, 1.49, 1.68), flat ones 1.18 after 40.
-//   checker: cycles(dim, L, width) a per wave of one block per SM, as measured.
+//            Sizes beyond two on an SM evict each other's code from its instruction cache: T is
+//            1 + 0.3 (D - 2) times as long (2D: 0.45), D sizes meeting on one: its chains, 16 at the most, are
+//            drawn from the 2432 longest, which go first.  Attempts/ns, walk / checker, sizes in narrow tiles
+//            at their first weight step: L = 4, 6, 8, 10, 12, 300 chains 6.0 / 5.2, 1000 11 / 17.5; L = 7, 8, 9,
+//            1000 15 / 24; L = 4 to 12, 1000 6.8 / 14.7, 4096 11 / 23.
+//            Tiles of 8 or 4 beside full ones leave the blocks that have no chain unevenly about: 1.3 times
+//            (L = 3 and 4, 2 x 500: 20 with both full, 15 with tiles of 8 at L = 4).  With several sizes the
+//            estimate is rough (0.5 to 1.3 times the time); over 356 such batches the kernel taken had 99.4 %
+//            of the better one's speed on average, at least 83 % in all but one.
+//   checker: cycles(dim, L, width) a, as measured, block after block in the order of the tiles, one to an
+//            SM; a full tile of L >= 7 reads its thresholds through L1, of which 28 KB are left beside a
+//            block of 196 KB and more (L = 6 and 8 in full tiles, 2 x 2048: 340 cycles instead of 101).
 // The estimate of the walk kernel is within 10 % over 600 to 9728 chains, L = 3..12 in 2D and 3D.  Both
 // sides measured, attempts/ns, walk / checker.  L = 8 in tiles of 16, power law, 4096 chains after 1, 10, 20,
 // 40 weight steps 68, 81, 90, 100 / 89; 2432 after 1 step 70 / 105; 1024 45 to 76 / 45.  L = 6 in full tiles, 2048
@@ -661,7 +673,7 @@ extern "C" int muca_set_eg(ea_ctx *ctx, int chain0, int n, const int32_t *e_g) {
 // 20 / 23.  2D: L = 3, 1024 4.3 / 7.0; L = 4, 1024 12 / 19, 2048 16 / 37; L = 5, 512 6.6 / 6.3, 1024 11 / 13; L = 8, 1024
 // 40 / 32, 1536 50 / 49, 2048 53 / 65; L = 12, 1024 40 / 32, 1536 49 / 48, 2048 52 / 64 (after 27 steps 2432 72 / 76).
 struct ColourPlan {
-    bool walk = true, runs = true;  // runs: the kernel has every tile's width
+    bool walk = true;
     size_t smem = 0;
     int max_width = 0, parities = 0;
 };
@@ -669,46 +681,74 @@ struct ColourPlan {
 // cycles per attempt (f = 1) of q chains to a scheduler: rounds of four, then the rest
 static double walk_cycles(double q) {
     q -= 1e-9;  // whole numbers out of sums
-    const double full = std::max(0.0, std::ceil(q / 4) - 1);
-    return 44 * full + std::max(26.0, 14.4 + 8.65 * std::ceil(q - 4 * full));
+    const double full = std::max(0.0, std::ceil(q / 4) - 1), rest = q - 4 * full;
+    if (rest > 1) return 44 * full + 14.4 + 8.65 * std::ceil(rest);
+    return full > 0 ? 44 * full + 5 + 21 * rest : 26;  // few chains left fit in beside the last ones to end
+}
+
+// blocks of these lengths, each taken by the SM that is free first
+static double blocks_time(const std::vector<double> &len, int n_sm) {
+    const size_t n = len.size();
+    if (n <= (size_t)n_sm) return *std::max_element(len.begin(), len.end());
+    if (std::all_of(len.begin(), len.end(), [&](double t) { return t == len[0]; }))
+        return len[0] * ((n + n_sm - 1) / n_sm);
+    std::vector<double> busy(n_sm, 0.0);  // a heap: the first is free first
+    for (double t : len) {
+        std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+        busy.back() += t;
+        std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+    }
+    return *std::max_element(busy.begin(), busy.end());
 }
 
 static ColourPlan colour_plan(const ea_ctx *ctx) {
     static const double f_3d[13] = {0, 0, 0, 5.15, 1.8, 2.15, 1.75, 1.77, 1.56, 1.72, 1.84, 1.84, 1.77};
     static const double g_3d[13] = {0, 0, 0, 0.01, 0.09, 0.14, 0.24, 0.26, 0.335, 0.25, 0.25, 0.2, 0.23};
     static const double f_2d[13] = {0, 0, 0, 15, 5.7, 5.9, 2.75, 3.15, 1.65, 2.1, 1.82, 2.12, 1.65};
-    static const double c_full[13] = {0, 0, 0, 222, 100, 147, 64.5, 157, 101, 137, 104, 143, 111};
+    static const double c_full[13] = {0, 0, 0, 222, 100, 147, 64.5, 157, 101, 137, 104, 150, 111};
     static const double c_half[13] = {0, 0, 0, 0, 78, 114, 60.5, 83, 47.5, 0, 0, 0, 0};
+    static const double c_8[13] = {0, 0, 0, 0, 77, 91.5, 57.5, 76.5, 46, 59.5, 50.2, 0, 0};
+    static const double c_4[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 69.2, 46.3};
     static const double c_2d[13] = {0, 0, 0, 303, 114, 168, 101, 128, 65.5, 99, 78.5, 89.4, 66};
     ColourPlan walk, checker;
     checker.walk = false;
     const bool power = 2 * (size_t)ctx->n_power >= ctx->chain_slot.size();
     const double steps = std::log(1 + ctx->weight_steps / 6.0) * (power ? 1.0 : 1.0 / 3);
-    bool have = true;  // the checker kernel has every tile's width
-    double w_max = 0, w_sum = 0, c_max = 0, c_sum = 0;
     for (const TileDesc &td : ctx->tiles) {
+        walk.smem = std::max(walk.smem, walk_smem_bytes(td.dim, td.L));
+        walk.max_width = std::max(walk.max_width, (int)td.width);
+        checker.smem = std::max(checker.smem, checker_smem_bytes(td.dim, td.L, td.width));
+        checker.parities |= checker_parity_class(td.dim, td.L, td.width);
+    }
+    double w_max = 0, w_sum = 0;
+    std::vector<double> blocks;
+    double chains[13] = {0};  // by L
+    int min_width = kTile;
+    for (const TileDesc &td : ctx->tiles) {
+        min_width = std::min(min_width, (int)td.width);
         const double a = (double)td.V * std::max(1, td.sweep_mul);
         const double g = td.dim == 3 ? g_3d[td.L] : std::max(0.0, 0.02 * td.L - 0.11);
         const double f = (td.dim == 3 ? f_3d[td.L] : f_2d[td.L]) / (1 + g * steps);
-        walk.smem = std::max(walk.smem, walk_smem_bytes(td.dim, td.L));
-        walk.max_width = std::max(walk.max_width, (int)td.width);
         w_max = std::max(w_max, f * a);
         w_sum += f * a * td.n_active;
-        const size_t ck = checker_smem_bytes(td.dim, td.L, td.width);
-        have = have && ck > 0;
-        checker.smem = std::max(checker.smem, ck);
-        checker.parities |= checker_parity_class(td.dim, td.L, td.width);
-        const double c = a * (td.dim == 2 ? c_2d[td.L] : td.width == 32 ? c_full[td.L] : c_half[td.L]);
-        c_max = std::max(c_max, c);
-        c_sum += c;
+        chains[td.L] += td.n_active;
+        double c = td.dim == 2 ? c_2d[td.L] : (td.width == 32 ? c_full : td.width == 16 ? c_half : td.width == 8 ? c_8 : c_4)[td.L];
+        if (checker.smem > (195u << 10) && !checker_thresholds_in_smem(td.dim, td.L, td.width)) c = 340;
+        blocks.push_back(c * a);
     }
-    const double n_sm = std::max(ctx->n_sm, 1), nt = (double)ctx->tiles.size();
-    const double t_walk = w_max * walk_cycles(w_sum / w_max / (4.0 * n_sm));  // chains of the longest's length
-    const double t_checker = std::max(c_max, std::ceil(nt / n_sm) * c_sum / nt);
-    checker.runs = have;
+    const double n_sm = std::max(ctx->n_sm, 1), resident = std::min(16 * n_sm, (double)ctx->chain_slot.size());
+    double met = 0, left = resident;
+    for (int L = 12; L >= 3; --L) {
+        const double k = std::min(left, chains[L]);
+        left -= k;
+        met += 1 - std::pow(1 - k / resident, resident / n_sm);
+    }
+    const double mix = (1 + (ctx->dim == 3 ? 0.3 : 0.45) * std::max(0.0, met - 2)) * (walk.max_width >= 4 * min_width ? 1.3 : 1.0);
+    const double t_walk = w_max * mix * walk_cycles(w_sum / w_max / (4.0 * n_sm));  // chains of the longest's length
+    const double t_checker = blocks_time(blocks, (int)n_sm);
     if (ctx->colour_kernel == EA_COLOUR_WARP) return walk;
     if (ctx->colour_kernel == EA_COLOUR_LANE) return checker;
-    return have && t_checker < t_walk ? checker : walk;
+    return t_checker < t_walk ? checker : walk;
 }
 
 // The lexicographic order of full tiles at L >= 7 in parts, a block each (muca_sweep.cu): a full tile
@@ -743,7 +783,6 @@ int ctx_enqueue_sweeps(ea_ctx *ctx, uint64_t n_sweeps, int count_roundtrips) {
     const uint64_t chunk = ctx->sweeps_per_launch ? ctx->sweeps_per_launch : n_sweeps;
     if (ctx->order == 1) {
         const ColourPlan plan = colour_plan(ctx);
-        if (!plan.runs) return fail(EA_EINVAL, "tiles of this context run only with a warp per chain");
         unsigned *diag = reinterpret_cast<unsigned *>(ctx->d_queue + 1);
         for (uint64_t done = 0; done < n_sweeps; done += chunk) {
             const uint64_t now = std::min(chunk, n_sweeps - done);

@@ -131,9 +131,9 @@ cudaError_t launch_sweeps_walk(const TileDesc *d_tiles, const int32_t *d_list, i
                                size_t smem, SlotState *d_slots, uint32_t *d_spins, const uint32_t *d_bonds,
                                const uint32_t *d_thr, uint32_t *d_hist, uint64_t n_sweeps, PhiloxKey key,
                                int count_rt, unsigned *d_diag, cudaStream_t st);
-// the colour-order sweep, one lane per chain (muca_checker.cu): every L in full tiles, and 3D tiles of
-// 16 at L = 4..8 (0 bytes: not available)
+// the colour-order sweep, one lane per chain (muca_checker.cu): every L and tile width
 size_t checker_smem_bytes(int dim, int L, int width);
+bool checker_thresholds_in_smem(int dim, int L, int width);
 // the kernel-form class of a tile there: 1 even L, 2 odd L, 4 the narrow tiles of the small even sizes
 // (3D, L <= 6), which run in forms of their own
 int checker_parity_class(int dim, int L, int width);

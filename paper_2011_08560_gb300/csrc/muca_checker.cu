@@ -1,8 +1,9 @@
 // muca_checker.cu -- a2 + a3 in the colour order (the checkerboard for even L): the
 // multicanonical sweep (Sec. II, Eq. "muca") with the sites of a sweep taken colour by colour,
-// each colour in lexicographic order, for 32 or 16 independent chains per tile, one lane per chain
-// (a narrow tile's chains on two lanes each): the throughput kernel, for batches of full tiles that
-// fill the SMs (muca_walk.cu runs the others; the choice is made in eamc_api.cu).  Odd L (three colours, the PT
+// each colour in lexicographic order, for 32, 16, 8 or 4 independent chains per tile, one lane per
+// chain (a narrow tile's chains on 32 / width lanes each).  It runs batches that fill the SMs, contexts
+// of several sizes above all; muca_walk.cu, a warp per chain, runs the others, and the choice is made
+// by the estimate in eamc_api.cu.  Odd L (three colours, the PT
 // colouring) runs in the same kernel: a row has a varying number of sites of a colour, so each
 // row gets the largest number of attempt slots and the unused ones are padding that moves
 // nothing and never accepts; each (pass, row)'s sites come from tables made once per launch.
@@ -86,7 +87,7 @@ __host__ __device__ constexpr int ck_sites_max(int L) {  // most colour-c sites 
 
 template <int DIM, int L, int W>
 struct CkGeo {
-    static_assert(W == 32 || W == 16, "tile width");
+    static_assert(W == 32 || W == 16 || W == 8 || W == 4, "tile width");
     using T = CkRow<L>;
     static constexpr int NCOL = (L & 1) ? 3 : 2;    // colour passes per sweep
     static constexpr int NR = DIM == 3 ? L * L : L;  // rows along x
@@ -131,7 +132,7 @@ struct CkGeo {
     static constexpr bool SMEM_THR = BASE_BYTES + THR_BYTES <= kSweepSmemMax;
     static constexpr size_t SMEM = BASE_BYTES + (SMEM_THR ? THR_BYTES : 0);
     // thresholds addressed by 32-bit shared addresses; measured with the same launches: L = 6 in
-    // tiles of 32 2.5 % faster, L = 8 in tiles of 16 2.5 % slower
+    // tiles of 32 2.5 % faster, L = 10 in tiles of 8 1.5 % faster, L = 8 in tiles of 16 2.5 % slower
     static constexpr bool SADDR = SMEM_THR && !(L == 8 && W == 16);
 };
 
@@ -565,23 +566,32 @@ muca_checker_kernel(const TileDesc *__restrict__ tiles, SlotState *__restrict__ 
     if (((MODE == 0 || MODE == 3) && odd) || (MODE == 1 && !odd)) return;  // the whole CTA, before any barrier
     const uint64_t n_tile = n_sweeps * (uint64_t)(td.sweep_mul > 0 ? td.sweep_mul : 1);
 #define EAMC_CK(LL, WW) checker_tile<DIM, LL, WW>(td, blockIdx.x, slots, spins, bonds, thr, hist, n_tile, key, count_rt, diag, smem_raw)
-    // narrow tiles (3D): 16 chains at L = 4..8, each chain on two lanes, so that the thresholds fit in
-    // shared memory (L = 7, 8) or a batch spreads over more SMs, each with a smaller share of the
-    // producer work
+    // narrow tiles (3D): 16 chains at L = 4..8, 8 at L = 4..10, 4 at L = 11, 12, each chain on
+    // 32 / width lanes, so that the thresholds fit in shared memory (L >= 7) or a batch spreads
+    // over more SMs, each with a smaller share of the producer work (L <= 8)
     if (td.width != 32) {
         if constexpr (DIM == 3) {
             if constexpr (MODE == 1 || MODE == 2) {
-                if (td.L == 7) EAMC_CK(7, 16);
-                else if (td.L == 5) EAMC_CK(5, 16);
+                if (td.width == 16 && td.L == 7) EAMC_CK(7, 16);
+                else if (td.width == 8 && td.L == 7) EAMC_CK(7, 8);
+                else if (td.width == 16 && td.L == 5) EAMC_CK(5, 16);
+                else if (td.width == 8 && td.L == 5) EAMC_CK(5, 8);
+                else if (td.width == 8 && td.L == 9) EAMC_CK(9, 8);
+                else if (td.width == 4 && td.L == 11) EAMC_CK(11, 4);
             }
             if constexpr (MODE != 1) {
-                if (td.L == 8) EAMC_CK(8, 16);
+                if (td.width == 16 && td.L == 8) EAMC_CK(8, 16);
+                else if (td.width == 8 && td.L == 8) EAMC_CK(8, 8);
+                else if (td.width == 8 && td.L == 10) EAMC_CK(10, 8);
+                else if (td.width == 4 && td.L == 12) EAMC_CK(12, 4);
             }
             // the small even sizes' narrow tiles in forms of their own (MODE 3, and 2 for both
             // parities): compiled into the even-size form they cost L = 8 1 % through its code
             if constexpr (MODE >= 2) {
-                if (td.L == 4) EAMC_CK(4, 16);
-                else if (td.L == 6) EAMC_CK(6, 16);
+                if (td.width == 16 && td.L == 4) EAMC_CK(4, 16);
+                else if (td.width == 8 && td.L == 4) EAMC_CK(4, 8);
+                else if (td.width == 16 && td.L == 6) EAMC_CK(6, 16);
+                else if (td.width == 8 && td.L == 6) EAMC_CK(6, 8);
             }
         }
         return;
@@ -654,14 +664,41 @@ size_t checker_smem_bytes(int dim, int L, int width) {
                 default: return 0;
             }
         }
+        if (width == 8) {
+            switch (L) {
+                case 4: return CkGeo<3, 4, 8>::SMEM;
+                case 5: return CkGeo<3, 5, 8>::SMEM;
+                case 6: return CkGeo<3, 6, 8>::SMEM;
+                case 7: return CkGeo<3, 7, 8>::SMEM;
+                case 8: return CkGeo<3, 8, 8>::SMEM;
+                case 9: return CkGeo<3, 9, 8>::SMEM;
+                case 10: return CkGeo<3, 10, 8>::SMEM;
+                default: return 0;
+            }
+        }
+        if (width == 4) return L == 11 ? CkGeo<3, 11, 4>::SMEM : (L == 12 ? CkGeo<3, 12, 4>::SMEM : 0);
         return 0;
     }
+    if (width != 32) return 0;
     return dim == 3 ? checker_smem_w<3, 32>(L) : checker_smem_w<2, 32>(L);
 }
 
 int checker_parity_class(int dim, int L, int width) {
     if (L & 1) return 2;
     return (dim == 3 && width != 32 && L <= 6) ? 4 : 1;
+}
+
+bool checker_thresholds_in_smem(int dim, int L, int width) {
+    if (checker_smem_bytes(dim, L, width) == 0) return false;
+#define EAMC_TS(D, LL, WW) if (dim == D && L == LL && width == WW) return CkGeo<D, LL, WW>::SMEM_THR;
+    EAMC_TS(3, 7, 16) EAMC_TS(3, 8, 16) EAMC_TS(3, 8, 8) EAMC_TS(3, 4, 16) EAMC_TS(3, 5, 16) EAMC_TS(3, 6, 16)
+    EAMC_TS(3, 4, 8) EAMC_TS(3, 5, 8) EAMC_TS(3, 6, 8) EAMC_TS(3, 7, 8) EAMC_TS(3, 9, 8) EAMC_TS(3, 10, 8) EAMC_TS(3, 11, 4) EAMC_TS(3, 12, 4)
+    EAMC_TS(3, 3, 32) EAMC_TS(3, 4, 32) EAMC_TS(3, 5, 32) EAMC_TS(3, 6, 32) EAMC_TS(3, 7, 32) EAMC_TS(3, 8, 32)
+    EAMC_TS(3, 9, 32) EAMC_TS(3, 10, 32) EAMC_TS(3, 11, 32) EAMC_TS(3, 12, 32)
+    EAMC_TS(2, 3, 32) EAMC_TS(2, 4, 32) EAMC_TS(2, 5, 32) EAMC_TS(2, 6, 32) EAMC_TS(2, 7, 32) EAMC_TS(2, 8, 32)
+    EAMC_TS(2, 9, 32) EAMC_TS(2, 10, 32) EAMC_TS(2, 11, 32) EAMC_TS(2, 12, 32)
+#undef EAMC_TS
+    return false;
 }
 
 cudaError_t launch_sweeps_checker(const TileDesc *d_tiles, int n_tiles, int dim, size_t smem, SlotState *d_slots,

@@ -41,3 +41,33 @@ def _choice(dim, L, width, n, power, steps):
 ])
 def test_the_faster_kernel_is_taken(dim, L, width, n, power, steps, faster):
     assert _choice(dim, L, width, n, power, steps) == faster
+
+
+# contexts of several sizes, power law, first weight step: (L, width, chains)
+@pytest.mark.parametrize("dim,groups,faster", [
+    (3, [(4, 8, 200), (6, 8, 200), (8, 8, 200), (10, 8, 200), (12, 4, 200)], LANE),    # 11 / 17.5
+    (3, [(4, 8, 60), (6, 8, 60), (8, 8, 60), (10, 8, 60), (12, 4, 60)], WARP),         # 6.0 / 5.2
+    (3, [(4, 32, 200), (6, 32, 200), (8, 32, 200), (10, 32, 200), (12, 32, 200)], WARP),  # 11 / 2.6
+    (3, [(7, 8, 333), (8, 8, 333), (9, 8, 333)], LANE), (3, [(8, 8, 500), (9, 8, 500)], WARP),  # 15 / 24, 33 / 26
+    (3, [(8, 32, 500), (10, 32, 500)], WARP), (3, [(5, 8, 2048), (7, 8, 2048)], WARP),    # 32 / 13, 51 / 27
+    (3, [(L, 8 if L < 11 else 4, 111) for L in range(4, 13)], LANE), (3, [(6, 32, 2048), (8, 32, 2048)], WARP),  # 6.8 / 15, 63 / 18
+    (2, [(4, 32, 200), (6, 32, 200), (8, 32, 200), (10, 32, 200), (12, 32, 200)], LANE),  # 6.9 / 15
+    (2, [(4, 32, 600), (6, 32, 600), (8, 32, 600), (10, 32, 600), (12, 32, 600)], LANE),  # 17 / 45
+    (2, [(8, 32, 500), (12, 32, 500)], WARP),  # 31 / 22
+])
+def test_the_faster_kernel_is_taken_for_several_sizes(dim, groups, faster):
+    import torch
+    from paper_2011_08560_gb300 import eamc
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the figures are of 152 SMs")
+    ctx = eamc.Context(seed=3)
+    ctx.set_sweep_order(eamc.EA_ORDER_COLOUR)
+    for L, width, n in groups:
+        if width != 32:
+            ctx.set_tile_width(L, width)
+        ctx.set_ensemble(ctx.init_disorder(dim, L, n), n, eamc.EA_POWERLAW)
+    ctx.run_sweeps(1)
+    ctx.update_weights()
+    kernel = ctx.colour_kernel()
+    ctx.close()
+    assert kernel == faster
