@@ -456,8 +456,7 @@ extern "C" int ea_init_disorder(ea_ctx *ctx, int dim, int L, int n, uint32_t rid
         ctx->chain_woff.push_back(nt[k / W].w_base + (uint64_t)(k % W) * B);
         ctx->chain_btop.push_back(0);
     }
-    ctx->chain_power.resize(ctx->chain_slot.size(), 0);
-    ctx->weight_steps = 0;
+    ctx->add_chains(n);
     if ((rc = ctx_refresh_chains(ctx))) return rc;
     if ((rc = ctx_rebuild_order(ctx))) return rc;
     // flat weights (ln W = 0 already) -> thresholds
@@ -502,7 +501,7 @@ extern "C" int muca_set_ensemble(ea_ctx *ctx, int chain0, int n, int kind, doubl
                                                                 pole_dE, beta);
     EA_CUDA(cudaGetLastError());
     EA_CUDA(cudaStreamSynchronize(ctx->stream));
-    for (int k = 0; k < n; ++k) ctx->set_power(chain0 + k, kind == EA_POWERLAW);
+    ctx->set_history(chain0, n, kind == EA_POWERLAW, -1);
     return EA_OK;
 }
 
@@ -571,11 +570,25 @@ static int table_io(ea_ctx *ctx, int chain0, int n, T *table, int width, T *host
     return EA_OK;
 }
 
+// the weight steps it takes to reach the given tables, read off 8 of the n rows (chain k's row is row(k)):
+// a step raises the weights of the bins that a chain has not reached yet against its top bin by the
+// logarithm of its counts there, 6.4 to 8.5 with 300 to 1500 sweeps a step (L = 6..12, either recursion)
+template <class Row, class Rise>
+static void steps_from_rows(ea_ctx *ctx, int chain0, int n, Row row, Rise rise) {
+    const int every = (n + 7) / 8;
+    for (int k0 = 0; k0 < n; k0 += every) {
+        const double r = rise(row(chain0 + k0), ctx->chain_btop[chain0 + k0]) / 7.0;
+        const int steps = r > 0 ? (int)std::min(r + 0.5, (double)ea_ctx::kMaxSteps) : 0;
+        ctx->set_history(chain0 + k0, std::min(every, n - k0), -1, steps);
+    }
+}
+static double weights_rise(const double *w, int b_top) { return *std::max_element(w, w + b_top + 1) - w[b_top]; }
+
 extern "C" int muca_set_weights(ea_ctx *ctx, int chain0, int n, const double *lnW, int stride) {
     int rc = table_io<double>(ctx, chain0, n, ctx ? ctx->d_lnW : nullptr, 1, const_cast<double *>(lnW),
                               stride, true);
     if (rc) return rc;
-    ctx->weights_given();
+    steps_from_rows(ctx, chain0, n, [&](int c) { return lnW + (size_t)(c - chain0) * stride; }, weights_rise);
     EA_CUDA(launch_quantize(ctx->d_tiles, (int)ctx->tiles.size(), ctx->d_slots, ctx->d_lnW, ctx->d_thr,
                             ctx->stream));
     return EA_OK;
@@ -595,7 +608,14 @@ extern "C" int muca_set_thresholds(ea_ctx *ctx, int chain0, int n, const uint32_
                                 stride, true);
     if (rc) return rc;
     ctx->thr_injected = true;
-    ctx->weights_given();
+    // a step up by one bin (dim - 1 unsatisfied bonds) is accepted with W(b + 1) / W(b) where that is below 1
+    const int up = ctx->dim - 1;
+    steps_from_rows(ctx, chain0, n, [&](int c) { return thr + (size_t)(c - chain0) * stride; },
+                    [&](const uint32_t *t, int b_top) {
+                        double rise = 0;
+                        for (int b = 0; b < b_top; ++b) rise -= std::log((t[8 * b + up] + 1.0) / 4294967296.0);
+                        return rise;
+                    });
     EA_CUDA(launch_enforce_walls(ctx->d_tiles, (int)ctx->tiles.size(), ctx->d_slots, ctx->d_thr, ctx->stream));
     EA_CUDA(cudaStreamSynchronize(ctx->stream));
     return EA_OK;
@@ -712,8 +732,15 @@ static ColourPlan colour_plan(const ea_ctx *ctx) {
     static const double c_2d[13] = {0, 0, 0, 303, 114, 168, 101, 128, 65.5, 99, 78.5, 89.4, 66};
     ColourPlan walk, checker;
     checker.walk = false;
-    const bool power = 2 * (size_t)ctx->n_power >= ctx->chain_slot.size();
-    const double steps = std::log(1 + ctx->weight_steps / 6.0) * (power ? 1.0 : 1.0 / 3);
+    // 1 / r of this g, over the chains
+    auto slowness = [&](double g) {
+        double sum = 0;
+        for (int power = 0; power < 2; ++power)
+            for (int s = 0; s <= ea_ctx::kMaxSteps; ++s)
+                if (ctx->history[power][s]) sum += ctx->history[power][s] / (1 + g * std::log(1 + s / 6.0) * (power ? 1.0 : 1.0 / 3));
+        return sum / (double)ctx->chain_slot.size();
+    };
+    double f_of[13] = {0};  // f / r by L
     for (const TileDesc &td : ctx->tiles) {
         walk.smem = std::max(walk.smem, walk_smem_bytes(td.dim, td.L));
         walk.max_width = std::max(walk.max_width, (int)td.width);
@@ -727,8 +754,9 @@ static ColourPlan colour_plan(const ea_ctx *ctx) {
     for (const TileDesc &td : ctx->tiles) {
         min_width = std::min(min_width, (int)td.width);
         const double a = (double)td.V * std::max(1, td.sweep_mul);
-        const double g = td.dim == 3 ? g_3d[td.L] : std::max(0.0, 0.02 * td.L - 0.11);
-        const double f = (td.dim == 3 ? f_3d[td.L] : f_2d[td.L]) / (1 + g * steps);
+        double &f = f_of[td.L];
+        if (f == 0)
+            f = td.dim == 3 ? f_3d[td.L] * slowness(g_3d[td.L]) : f_2d[td.L] * slowness(std::max(0.0, 0.02 * td.L - 0.11));
         w_max = std::max(w_max, f * a);
         w_sum += f * a * td.n_active;
         chains[td.L] += td.n_active;
@@ -949,6 +977,7 @@ extern "C" int ea_graph_capture(ea_ctx *ctx, int n_iter, uint64_t sweeps_per_ite
     uint64_t mul = 1;
     for (const TileDesc &td : ctx->tiles) mul = std::max<uint64_t>(mul, (uint64_t)td.sweep_mul);
     ctx->graph_sweeps = (uint64_t)n_iter * sweeps_per_iter * mul;
+    ctx->graph_steps = update_weights ? n_iter : 0;
     return EA_OK;
 }
 
@@ -960,6 +989,7 @@ extern "C" int ea_graph_launch(ea_ctx *ctx, int replays) {
         return fail(EA_EINVAL, "sweep counter would exceed 2^32");
     for (int r = 0; r < replays; ++r) EA_CUDA(cudaGraphLaunch(ctx->graph_exec, ctx->stream));
     ctx->max_t_host += (uint64_t)replays * ctx->graph_sweeps;
+    ctx->step_all((int)std::min<int64_t>((int64_t)replays * ctx->graph_steps, ea_ctx::kMaxSteps));
     return EA_OK;
 }
 
@@ -978,7 +1008,7 @@ extern "C" int muca_update_weights(ea_ctx *ctx) {
     const int nt = (int)ctx->tiles.size();
     EA_CUDA(launch_update_weights(ctx->d_tiles, nt, ctx->d_slots, ctx->d_lnW, ctx->d_hist, ctx->d_acc, ctx->stream));
     EA_CUDA(launch_quantize(ctx->d_tiles, nt, ctx->d_slots, ctx->d_lnW, ctx->d_thr, ctx->stream));
-    ctx->weight_steps = std::min(ctx->weight_steps + 1, ea_ctx::kIteratedSteps);
+    ctx->step_all(1);
     return EA_OK;
 }
 
@@ -1005,8 +1035,7 @@ extern "C" int muca_build_ensemble(ea_ctx *ctx, int chain0, int n, int kind, dou
     const int nt = (int)ctx->tiles.size();
     EA_CUDA(launch_build_ensemble(ctx->d_tiles, nt, ctx->d_slots, d_sel, kind, alpha, pole_dE, beta,
                                   ctx->d_lnW, ctx->stream));
-    for (int k = 0; k < n; ++k) ctx->set_power(chain0 + k, kind == EA_POWERLAW);
-    ctx->weights_given();
+    ctx->set_history(chain0, n, kind == EA_POWERLAW, -1);
     // the other chains' thresholds are those of their weights already, unless injected ones are about
     // (2304 chains of L = 6, 128 of them built: 0.12 -> 0.01 ms a call)
     if (ctx->thr_injected) {
@@ -1058,6 +1087,7 @@ extern "C" int ea_reset_chains(ea_ctx *ctx, const int32_t *chains, int n, const 
     int herr = 0;
     EA_CUDA(cudaMemcpyAsync(&herr, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     EA_CUDA(cudaStreamSynchronize(ctx->stream));
+    for (int k = 0; k < n; ++k) ctx->set_history(chains[k], 1, -1, 0);
     if ((rc = ctx_refresh_chains(ctx))) return rc;
     if (herr) return fail(EA_ESTATE, "descent to E_top got stuck for a reset chain (left inactive)");
     return EA_OK;
@@ -1072,6 +1102,7 @@ extern "C" int muca_update_weights_subset(ea_ctx *ctx, const int32_t *chains, in
     int rc = upload_slots(ctx, chains, n, 0, &scr, &d_slot);
     if (rc) return rc;
     EA_CUDA(launch_update_weights_sel(ctx->d_tiles, ctx->d_slots, ctx->d_lnW, ctx->d_hist, ctx->d_acc, d_slot, n, ctx->stream));
+    for (int k = 0; k < n; ++k) ctx->set_history(chains[k], 1, -1, ctx->chain_steps[chains[k]] + 1);
     EA_CUDA(launch_quantize(ctx->d_tiles, (int)ctx->tiles.size(), ctx->d_slots, ctx->d_lnW, ctx->d_thr,
                             ctx->stream));
     EA_CUDA(cudaStreamSynchronize(ctx->stream));
@@ -1130,7 +1161,7 @@ extern "C" int muca_copy_weights(ea_ctx *ctx, const int32_t *src, const int32_t 
     int32_t *d_meta = (int32_t *)((char *)scr + ((off.size() * 8 + 255) & ~(size_t)255));
     EA_CUDA(cudaMemcpyAsync(d_off, off.data(), off.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
     EA_CUDA(cudaMemcpyAsync(d_meta, meta.data(), meta.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
-    ctx->weights_given();
+    for (int k = 0; k < n; ++k) ctx->set_history(dst[k], 1, ctx->chain_power[src[k]], ctx->chain_steps[src[k]]);
     copy_weights_kernel<<<n, 128, 0, ctx->stream>>>(ctx->d_slots, ctx->d_lnW, d_meta, d_off, n);
     EA_CUDA(cudaGetLastError());
     EA_CUDA(launch_quantize(ctx->d_tiles, (int)ctx->tiles.size(), ctx->d_slots, ctx->d_lnW, ctx->d_thr,
@@ -1350,14 +1381,20 @@ extern "C" int ea_snapshot_load(ea_ctx *ctx, const void *buf, size_t size) {
     ctx->max_V = h.max_V;
     ctx->sweep_smem = h.sweep_smem;
     ctx->thr_injected = true;  // a snapshot may hold injected thresholds
-    ctx->weights_given();
-    ctx->chain_power.assign(h.n_chains, 0);
-    ctx->n_power = 0;
+    ctx->add_chains(h.n_chains);
+    const char *lnw = slots + h.n_tiles * kTile * sizeof(SlotState) + (h.spin_used + h.bond_used) * 4;
+    std::vector<double> row;
     for (size_t c = 0; c < h.n_chains; ++c) {
         if (cslot[c] < 0 || (size_t)cslot[c] >= h.n_tiles * kTile) continue;
         SlotState s;
         std::memcpy(&s, slots + (size_t)cslot[c] * sizeof(SlotState), sizeof s);
-        ctx->set_power((int)c, s.kind == EA_POWERLAW);
+        ctx->set_history((int)c, 1, s.kind == EA_POWERLAW, -1);
     }
+    steps_from_rows(ctx, 0, (int)h.n_chains, [&](int c) {
+        row.assign(std::max(1, cbtop[c] + 1), 0.0);
+        if (cbtop[c] >= 0 && cwoff[c] + cbtop[c] < h.w_used)
+            std::memcpy(row.data(), lnw + cwoff[c] * sizeof(double), row.size() * sizeof(double));
+        return row.data();
+    }, [](const double *w, int b_top) { return b_top >= 0 ? weights_rise(w, b_top) : 0.0; });
     return ctx_rebuild_order(ctx);
 }

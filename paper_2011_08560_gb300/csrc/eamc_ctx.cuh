@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <vector>
 
@@ -20,16 +21,43 @@ struct ea_ctx {
     uint64_t max_t_host = 0;  // upper bound of every chain's sweep counter
     bool thr_injected = false;  // some chain's thresholds may not be its weights' (muca_set_thresholds,
                                 // a snapshot): the next re-quantisation takes every chain
-    // what the colour order's choice of kernel goes by (speed only): the power-law chains, and the weight
-    // steps since the newest chains were made, given weights counted as kIteratedSteps of them
-    std::vector<uint8_t> chain_power;
-    int n_power = 0, weight_steps = 0;
-    static constexpr int kIteratedSteps = 40;
-    void set_power(int chain, bool power) {
-        n_power += (int)power - (int)chain_power[chain];
-        chain_power[chain] = power;
+    // what the colour order's choice of kernel goes by (speed only): of each chain, whether its ensemble is
+    // a power law, and the weight steps that its weights have been through (kMaxSteps at the most).  Steps
+    // count where they are queued, also those of a graph replay; weights and thresholds that are given, and
+    // those of a snapshot, count as the steps it takes to reach them.  Not counted: a server's own chains
+    // (taken as flat ones without a step), whose batches run a warp per chain unless lanes are many; and a
+    // captured graph keeps the kernel of its capture
+    static constexpr int kMaxSteps = 40;
+    std::vector<uint8_t> chain_power, chain_steps;
+    int history[2][kMaxSteps + 1] = {};  // chains by both
+    void add_chains(size_t n) {
+        chain_power.resize(chain_power.size() + n, 0);
+        chain_steps.resize(chain_steps.size() + n, 0);
+        history[0][0] += (int)n;
     }
-    void weights_given() { weight_steps = std::max(weight_steps, kIteratedSteps); }
+    // of the n chains from chain0 on; power or steps -1: as they are
+    void set_history(int chain0, int n, int power, int steps) {
+        steps = std::min(steps, kMaxSteps);
+        for (int c = chain0, end = chain0 + n; c < end;) {
+            const int p = chain_power[c], s = chain_steps[c], first = c;
+            const int p1 = power < 0 ? p : power, s1 = steps < 0 ? s : steps;
+            for (; c < end && chain_power[c] == p && chain_steps[c] == s; ++c) {
+                chain_power[c] = (uint8_t)p1;
+                chain_steps[c] = (uint8_t)s1;
+            }
+            history[p][s] -= c - first;
+            history[p1][s1] += c - first;
+        }
+    }
+    void step_all(int steps) {
+        steps = std::min(steps, kMaxSteps);
+        for (uint8_t &s : chain_steps) s = (uint8_t)std::min<int>(s + steps, kMaxSteps);
+        for (int (&h)[kMaxSteps + 1] : history)
+            for (int s = kMaxSteps - 1; s >= 0 && steps > 0; --s) {
+                h[std::min(s + steps, kMaxSteps)] += h[s];
+                h[s] = 0;
+            }
+    }
 
     // host mirrors
     std::vector<eamc::TileDesc> tiles;
@@ -68,6 +96,7 @@ struct ea_ctx {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t graph_exec = nullptr;
     uint64_t graph_sweeps = 0;        // sweeps one replay adds to every chain
+    int graph_steps = 0;              // and weight steps
 
     PtState *pt = nullptr;
 };
