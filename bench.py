@@ -56,10 +56,10 @@ LATENCY_FLOOR_CYCLES = {"colour": 6.4, "lex": 35.4}
 # 40 ops, 5 ops per plane) and the flip: about 150 lane-operations per 32 attempts
 PT_ALG_OPS = 4.7
 # dram__bytes_read.sum + dram__bytes_write.sum of one production launch of the headline workload
-# (L=8, 1024 chains, warp-per-chain kernel), ncu capture of this kernel version: 6.42 MB + 0 B for a
-# 2000-sweep launch.  It is the one-time staging of lattices and of the tables' parts around each
-# chain's bins, so it hardly grows with the sweeps of a launch.
-SWEEP_TRAFFIC_BYTES = 6.42e6
+# (L=8, 1024 chains, warp-per-chain kernel), ncu capture of this kernel version: 9.10 MB + 0 B for a
+# 2000-sweep launch of iterated chains.  It is the staging of lattices and of the tables' parts around
+# each chain's bins (the tables are 12.6 MB in all), so it hardly grows with the sweeps of a launch.
+SWEEP_TRAFFIC_BYTES = 9.10e6
 
 
 # what goes to the output line; everything else (the secondary workloads above all) only into the file
@@ -727,9 +727,8 @@ def build_uneven(eamc, autotune, stream_ptr, S: int, order: int = 0):
 def bench_uneven(S: int = 100, iters: int = 3, order: int = 0):
     """Uneven batch: 4096 realizations, L uniform over {4,6,8,10,12} (round robin by id), each
     as a power-law, a flat and a 1/k chain, in one launch per step (lexicographic order: the
-    persistent work-queue kernel; checkerboard order: one warp per chain, or one block
-    per tile where full tiles fill the GPU); the
-    weight-iteration loop is a captured CUDA graph."""
+    persistent work-queue kernel; checkerboard order: one block per tile, or one warp per
+    chain); the weight-iteration loop is a captured CUDA graph."""
     import torch
 
     from paper_2011_08560_gb300 import autotune, eamc

@@ -157,9 +157,11 @@ int muca_set_launch(ea_ctx *ctx, int persistent, uint64_t sweeps_per_launch, int
  *   c(x) = x mod 3 except c(L-1) = 1 when L = 1 (mod 3)), each in lexicographic order; the
  *   j-th colour-c site of a row takes word j&3 of call (4 row + j/4, t, rid, (5 + c) | stream << 8).
  *   No two sites of a class are neighbours, so each attempt's class is fixed when its class
- *   begins.  Two kernels run it, for every L, with the same results: one warp per chain, and one
- *   lane per chain for batches of full tiles that fill the GPU; the library takes the one it
- *   estimates to be faster for the context's tiles.  The faster order for small and middle batches.
+ *   begins.  Two kernels run it, for every L and tile width, with the same results: one warp per
+ *   chain, and one lane per chain; the library takes the one it estimates to be faster for the
+ *   context (muca_set_colour_kernel): a lane per chain for many chains, above all in their first weight
+ *   steps or in flat ensembles, and for several sizes at once.  The faster order for small and middle
+ *   batches.
  * chains_per_cta: 0 or one of 1, 2, 4, 8 (kept for callers of an earlier form of this call; it
  * has no effect).  Applies from the next muca_run_sweeps or graph capture; the order is not part
  * of a snapshot.  EA_EINVAL for an unknown order or count. */
@@ -167,7 +169,8 @@ int muca_set_sweep_order(ea_ctx *ctx, int order, int chains_per_cta);
 
 /* a2 -- the kernel that runs the colour order in this context: EA_COLOUR_AUTO (the default) takes the
  * one that the library estimates to be faster; EA_COLOUR_WARP is one warp per chain, EA_COLOUR_LANE
- * one lane per chain.  Results do not depend on it.
+ * one lane per chain.  Results do not depend on it.  Applies from the next muca_run_sweeps or graph
+ * capture; a captured graph keeps its kernel.
  * muca_get_colour_kernel: the kernel that the next muca_run_sweeps in the colour order takes. */
 #define EA_COLOUR_AUTO 0
 #define EA_COLOUR_WARP 1
@@ -182,8 +185,9 @@ int muca_get_colour_kernel(ea_ctx *ctx, int *kernel);
  * lexicographic order a tile is one warp; with width W < 32 each of its W chains runs on 32/W lanes
  * side by side, so the tile needs W/32 of the shared memory of a full one: at L >= 7 the acceptance
  * thresholds then fit in shared memory instead of being read through L1.  In the colour order the
- * width matters little: a chain has a warp of its own unless the batch fills the GPU.  Narrow tiles
- * suit batches with fewer chains than the GPU can hold; results do not depend on the width.
+ * width matters where a chain has a lane and not a warp of its own: there narrow tiles also spread a
+ * batch over more SMs.  Narrow tiles suit batches with fewer chains than the GPU can hold; results do
+ * not depend on the width.
  * EA_EINVAL for a width not available at this L. */
 int muca_set_tile_width(ea_ctx *ctx, int L, int width);
 

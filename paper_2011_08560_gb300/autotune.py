@@ -1,18 +1,20 @@
 """Self-written autotuner for the batched MUCA sweep launch (a8).
 
 Knobs:
-  * chains per tile for each lattice size (muca_set_tile_width): 32, or the narrow width that
-    brings the acceptance thresholds into shared memory (16 at L = 7, 8; in the colour order also
-    8 at L = 9, 10 and 4 at L = 11, 12).  A narrow tile runs each of
+  * chains per tile for each lattice size (muca_set_tile_width): 32, or a narrow width (16 at L = 7,
+    8, which brings the acceptance thresholds into shared memory; in the colour order 16 at L = 4..8,
+    8 at L = 4..10 and 4 at L = 11, 12).  A narrow tile runs each of
     its chains faster but holds half as many, so it wins when the batch is smaller than what the
     GPU can hold and loses when tiles queue for SMs;
   * the persistent work-queue grid vs one block per tile, and the resident blocks per SM of the
     persistent grid (chains are latency-bound, so tiles sharing an SM sub-partition slow each
     other down);
   * sweeps per launch.
-In the colour order (muca_set_sweep_order) only the tile width is tuned; it decides little there, since
-a chain has a warp of its own unless the batch fills the GPU with full tiles.  The order itself is the caller's choice (it changes
-the trajectories), never the tuner's.
+In the colour order (muca_set_sweep_order) only the tile width is tuned.  The candidates' chains are
+new ones with unit weights, which the library may sweep with another kernel than the caller's chains
+after some weight steps (a lane per chain against a warp per chain, which no width slows): the width is
+the best one of the first steps.  The order itself is the caller's choice (it changes the trajectories),
+never the tuner's.
 A candidate is timed with CUDA events on a scratch context with the same composition of chains
 (same dim, L and chain counts, a different seed), so tuning never advances the caller's chains,
 whose results do not depend on the choice anyway.  The winner is cached in a JSON file keyed by

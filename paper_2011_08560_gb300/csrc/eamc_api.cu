@@ -914,7 +914,7 @@ extern "C" int muca_set_tile_width(ea_ctx *ctx, int L, int width) {
     const int dim = ctx->dim ? ctx->dim : 3;
     if (!sweep_width_supported(dim, L, width) && !colour_width_supported(dim, L, width))
         return fail(EA_EINVAL, "tile width %d is not available for dim=%d, L=%d (32 always; in 3D 16 for "
-                               "L=7,8, and in the colour order 8 for L=9,10 and 4 for L=11,12)", width, dim, L);
+                               "L=7,8, and in the colour order 16 for L=4..8, 8 for L=4..10 and 4 for L=11,12)", width, dim, L);
     ctx->tile_width[L] = width;
     return EA_OK;
 }

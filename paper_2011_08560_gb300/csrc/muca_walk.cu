@@ -1,8 +1,9 @@
 // muca_walk.cu -- a2 + a3 in the colour order (the checkerboard for even L), one warp per chain:
 // the multicanonical sweep (Sec. II, Eq. "muca") with the sites of a sweep taken colour by colour,
 // each colour in lexicographic order.  It serves every L (3..12), 2D and 3D, and tiles of any
-// width; batches that fill the GPU with full tiles run in muca_checker.cu (the choice is made in
-// eamc_api.cu).
+// width; batches that the estimate in eamc_api.cu finds faster with a lane per chain run in
+// muca_checker.cu: many chains, and contexts of several sizes, whose code the chains of an SM would
+// evict from one another's instruction cache.
 //
 // What bounds it.  A chain is a serial chain of decisions: attempt i+1's threshold is thr[b][n] at
 // the bin b that attempt i leaves.  A kernel that loads the threshold for that bin pays a
@@ -16,17 +17,18 @@
 // The walk is parallel as well.  The batch's 32 attempts are four segments of eight; the eight
 // lanes of a segment start it from the eight positions around the current one (p - 4 .. p + 3), so
 // the four segments are walked at once, and a chain of three byte selects (segment 0 from p, each
-// next one from the end of the one before) picks the lanes whose start was right.  A segment whose
-// start is not among its eight candidates, or that leaves the window, ends the batch there: the
-// attempts before it count, the next batch begins after them.  On cold chains 28 of 32 attempts
-// count on average.  While a batch is walked, the masks of the next one are made for the same
+// next one from the end of the one before) picks the lanes whose start was right.  Where a segment's
+// start is not among its eight candidates, the attempts before it count (28 of 32 on average on cold
+// chains) and the rest of the batch is walked again, with the same masks, from candidates around
+// their end.  A batch ends early only where the walk comes to the window's end: the next one begins
+// after the attempts that count, in a new window.  While a batch is walked, the masks of the next one are made for the same
 // window; the window moves when the position comes near its end.  The bins outside the table are 0
 // (never accepted), so a wall needs no test.
 //
 // L = 8, 1024 power-law chains in production: 112.6 -> 69 ms per 10^4 sweeps (46.6 -> 76 attempts
 // per ns; 45.5 -> 28 cycles per attempt of a chain, 22 where a chain has a scheduler to itself);
 // 500 chains of L = 7: 13.6 -> 34 attempts/ns, 300 of L = 10 in full tiles 6.5 -> 19.  One warp
-// per chain costs about 11 warp instructions per attempt, so that beyond two chains per scheduler
+// per chain costs 8 to 10 warp instructions per attempt, so that beyond two chains per scheduler
 // the issue slots and the half-rate integer pipe are the bound (4096 chains: 109 attempts/ns, pipe
 // 68 % and issue 72 % busy).
 // Measured and left out: 32 bins instead of 24 (-5 %), 20 bins (within 1 %), the masks from fp16
@@ -35,7 +37,7 @@
 // segments of 16 with 16 candidates for hot chains (-10 %), two to eight chains per warp (longer
 // chains: 47 to 130 cycles per attempt), masks made after the walk instead of beside it (-10 %).
 //
-// Shared memory of a warp (7 KB at L = 8): the chain's lattice as row words (a nibble per site:
+// Shared memory of a warp (5.8 KB at L = 8, 8 KB at the most, L = 11): the chain's lattice as row words (a nibble per site:
 // spins; bonds Jx, Jy, Jz at bits 0, 1, 2), a pass's attempts {random word, entry} (a chunk of 32 or
 // 64 rows where a pass has more than 256), 64 bins of the threshold table class by class (reloaded
 // around the current bin when the window leaves them), the masks of two batches.

@@ -370,8 +370,10 @@ extern "C" int ea_srv_create(ea_srv **out, int device, void *cuda_stream, uint64
     if (rc) { delete s; return rc; }
     if ((rc = muca_set_sweep_order(s->ctx, cfg->sweep_order, 0))) { ea_destroy(s->ctx); delete s; return rc; }
     if (cfg->sweep_order == EA_ORDER_COLOUR) {
-        // the narrowest tiles whose thresholds fit in shared memory: each served chain runs as
-        // fast as it can (jobs are few per lattice size), the pool holds fewer lanes per tile
+        // the narrowest tiles: jobs are few per lattice size, so the pool grows by few lanes at a time,
+        // and where lanes are many and the sizes too (a lane per chain then) narrow tiles are the faster
+        // ones.  All running, attempts/ns with a lane per chain against a warp per chain: L = 4 to 12,
+        // 1000 jobs 19.1 against 4.9, 400 jobs 8.4 against 8.8, 96 jobs 2.0 against 3.8
         for (int L : s->Ls)
             for (int w : {4, 8, 16})
                 if (muca_set_tile_width(s->ctx, L, w) == EA_OK) break;
